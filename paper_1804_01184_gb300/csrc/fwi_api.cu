@@ -25,6 +25,7 @@
 #include "fwi_kernels.cuh"
 #include "fwi_stream.cuh"
 #include "fwi_warp.cuh"
+#include "fwi_resident.cuh"
 
 namespace {
 
@@ -309,7 +310,7 @@ int cuda_fail(cudaError_t e, const char *what)
 
 // Model, sponge tables and acquisition geometry (S1, S2).
 int setup(const Plan &P, const fwi_grid *g, int pz, const float *xa, const float *xb,
-          const fwi_sources *src, const fwi_receivers *rec, void *work, cudaStream_t st)
+          const fwi_sources *src, const fwi_receivers *rec, void *work, cudaStream_t st, bool adjoint = false)
 {
     TraceRange tr(PH_MODEL_BUILD);
     const fwi::Dims &d = P.d;
@@ -333,8 +334,9 @@ int setup(const Plan &P, const fwi_grid *g, int pz, const float *xa, const float
     if (rec->nr > 0) {
         LAUNCH(fwi::k_geometry, (rec->nr + 127) / 128, 128, 0, st, rec->xy, rec->nr, d, g->dx, 1.0,
                at<long long>(work, P.ridx), at<float>(work, P.rw), status);
-        LAUNCH(fwi::k_receiver_chain, (4 * rec->nr + 127) / 128, 128, 0, st, at<long long>(work, P.ridx), 4 * rec->nr,
-               at<int>(work, P.rl));
+        if (adjoint)   // only injection reads the chains
+            LAUNCH(fwi::k_receiver_chain, (4 * rec->nr + 127) / 128, 128, 0, st, at<long long>(work, P.ridx), 4 * rec->nr,
+                   at<int>(work, P.rl));
     }
     return FWI_OK;
 }
@@ -665,6 +667,12 @@ int plan_for(Plan &P, const fwi_grid *g, fwi_op op, int ns, int nr, size_t work_
     return FWI_OK;
 }
 
+}  // namespace
+
+#include "fwi_resident.inc"
+
+namespace {
+
 // Forward over all steps for one group, used by model, adjoint and gradient.
 //   traces: [bg][nr][nt] output or null.
 //   with_hist: keep the pressure history of the last segment (it is the pressure state of those
@@ -676,6 +684,18 @@ int forward_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const Fwd f{P, work, st, wav};
     const size_t bf = (size_t)bg * P.d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * P.d.Np;   // floats between snapshot slots
+    ResPlan rp;
+    if (res_wanted(P, bg, rp)) {
+        const int C = with_hist ? P.C : P.nt;
+        for (int n0 = 0; n0 < P.nt; n0 += C) {
+            const int n1 = std::min(n0 + C, P.nt);
+            const int rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, n0 / C),
+                                       n1 < P.nt ? res_checkpoint(P, work, n1 / C) : ResState{},
+                                       with_hist && n1 == P.nt ? at<float>(work, P.snap) : nullptr, traces);
+            if (rc) return rc;
+        }
+        return FWI_OK;
+    }
     const int last0 = with_hist ? (P.nseg - 1) * P.C : P.nt + 1;
     float *snap = with_hist ? at<float>(work, P.snap) : nullptr;
     auto pbuf = [&](int n) -> float * {
@@ -741,12 +761,19 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
         const int n0 = k * P.C, n1 = std::min(n0 + P.C, P.nt);
         if (k < P.nseg - 1) {   // recompute the segment from its checkpoint
             TraceRange tr(PH_RECOMPUTE);
-            const float *ck = at<float>(work, P.ckpt) + (size_t)k * 3 * slot;
-            CK(cudaMemcpyAsync(snap, ck, bf, cudaMemcpyDeviceToDevice, st));
-            CK(cudaMemcpyAsync(at<float>(work, P.vx[n0 & 1]), ck + slot, bf, cudaMemcpyDeviceToDevice, st));
-            CK(cudaMemcpyAsync(at<float>(work, P.vz[n0 & 1]), ck + 2 * slot, bf, cudaMemcpyDeviceToDevice, st));
-            for (int n = n0; n < n1; ++n)
-                f.step(n, s0, bg, snap + (size_t)(n - n0) * slot, snap + (size_t)(n + 1 - n0) * slot);
+            ResPlan rp;
+            if (res_wanted(P, bg, rp)) {
+                const int rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, k), ResState{}, snap,
+                                           nullptr);
+                if (rc) return rc;
+            } else {
+                const float *ck = at<float>(work, P.ckpt) + (size_t)k * 3 * slot;
+                CK(cudaMemcpyAsync(snap, ck, bf, cudaMemcpyDeviceToDevice, st));
+                CK(cudaMemcpyAsync(at<float>(work, P.vx[n0 & 1]), ck + slot, bf, cudaMemcpyDeviceToDevice, st));
+                CK(cudaMemcpyAsync(at<float>(work, P.vz[n0 & 1]), ck + 2 * slot, bf, cudaMemcpyDeviceToDevice, st));
+                for (int n = n0; n < n1; ++n)
+                    f.step(n, s0, bg, snap + (size_t)(n - n0) * slot, snap + (size_t)(n + 1 - n0) * slot);
+            }
         }
         TraceRange tr(PH_ADJOINT);
         for (int n = n1 - 1; n >= n0; --n) {
@@ -816,7 +843,7 @@ int adjoint_impl(const fwi_grid *g, int pz, const float *xa, const float *xb, co
     Plan P;
     int rc = plan_for(P, g, op, src->ns, rec->nr, work_bytes);
     if (rc) return rc;
-    if ((rc = setup(P, g, pz, xa, xb, src, rec, work, st))) return rc;
+    if ((rc = setup(P, g, pz, xa, xb, src, rec, work, st, true))) return rc;
     if ((rc = clear_acc(P, work, st))) return rc;
     const long long per_shot = (long long)P.nr * P.nt;
     for (int gi = 0; gi < P.ngroups; ++gi) {
@@ -1004,6 +1031,7 @@ int fwi_status(void *work, void *stream)
     CK(cudaStreamSynchronize(st));
     if (h & fwi::ST_EINVAL) return fail(FWI_EINVAL, "a contrast has 1 + xi <= 0 or a position lies outside the physical grid");
     if (h & fwi::ST_ECFL) return fail(FWI_ECFL, "dt exceeds the stability limit of the stencil for this model");
+    if (h & fwi::ST_ETIMEOUT) return fail(FWI_ETIMEOUT, "a bounded wait between the tiles of an on-chip launch expired");
     if (h & fwi::ST_EBOUNDS)
         return fail(FWI_EINVAL, "a bounds check of the checked build caught an out-of-range access (skipped)");
     return FWI_OK;

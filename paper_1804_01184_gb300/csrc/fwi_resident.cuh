@@ -1,0 +1,564 @@
+// fwi_resident.cuh -- time-step kernels that keep the wavefield on chip (sm_103a).
+//
+// A launch advances some shots by many steps.  Each shot's grid is cut into tx x tz tiles, one
+// CTA a tile, all CTAs of the launch resident at once (cooperative launch).  Global memory sees
+// only what the caller asked for (pressure history, traces, final state) and the tiles'
+// boundary exchange.
+//
+// Layout.  A warp owns R rows of its tile, a lane one float4 of columns of each: lane l holds
+// column group l - 1 (4 columns), so lanes 1 .. ng are the tile's own groups (at most 30) and
+// lanes 0 and ng + 1 the groups beside it.  The cells' fields and model sit in registers for the
+// whole launch.  The x-stencil of p reads shared rows, that of v_x shuffles within the warp, and
+// the z-stencils read the rows of other warps from shared memory.  The tile's rows are
+// extended by the M rows above and M - 1 below whose v_z the divergence of its own rows reads.
+//
+// One exchange a step: the halo's velocities are updated here too (the neighbours compute the
+// same values from the same operands), so only pressure crosses tiles, 2M - 1 cells deep.
+// Neighbours send each value as an 8-byte word (step tag, float) into the receiver's mailbox
+// in global memory (L2); the receiver polls the words themselves, so a step waits for one
+// store-to-load latency, without flags or fences.  Two mailbox slots alternate: a CTA sends
+// step n + 2 only after it has the neighbour's step n + 1, which the neighbour computed after
+// reading step n.
+//
+// Every cell's arithmetic is the streaming kernels' (fwi_warp.cuh), operation for operation, so
+// results are bitwise theirs for every tiling.
+#pragma once
+#include "fwi_warp.cuh"
+
+namespace fwi {
+
+constexpr int RES_RC = 64;      // receivers of a tile listed in shared memory
+// a wait gives up after this many polls (a poll is an L2 round trip, ~1 us: a few seconds)
+constexpr int RES_SPIN = 1 << 21;
+enum : int { ST_ETIMEOUT = 16 };
+
+// Shape of a resident CTA: up to NW warps of R rows of 30 column groups.
+template <int M_, int R_, int NW_>
+struct ResShape {
+    static constexpr int M = M_, R = R_, NW = NW_;
+    static constexpr int HR = 2 * M - 1;             // depth of the pressure halo
+    static constexpr int G = 30, W = 4 * G;          // own column groups, columns
+    static constexpr int E = NW * R, H = E - HR;     // extended rows (from -M on), own rows
+    static constexpr int PP = W + 16;                // pitch of a p row: column c at c + 8
+    static constexpr int PZ = 128;                   // pitch of a v_z row: lane l at 4 l
+    // mailbox slot, in words: 2M - 1 rows from above and below, 8 columns from the left and right
+    static constexpr int MB = HR * W, ML = 2 * HR * W, MR = ML + 8 * H, SLOT = MR + 8 * H;
+    // two slots and a ring of 4 for the lower right diagonal tile's first cell (diagonal tiles
+    // do not wait on each other)
+    static constexpr int MAIL = 2 * SLOT + 4;
+};
+
+// Four rows a warp (five at 4th order, whose windows are shorter): 96 registers of fields and model a thread and room for the stencil windows
+// (eight rows, 255 registers, 8 warps an SM: 4.9 us a step against 3.4 us; two rows, 20 warps: 3.9 us).
+using ResFwd2 = ResShape<2, 5, 12>;
+using ResFwd4 = ResShape<4, 4, 12>;
+
+// Cut of a shot's grid: tx x tz tiles; the first grem (hrem) tiles have one column group (row)
+// more than gbase (hbase).
+struct ResCut {
+    int tx, tz, gbase, grem, hbase, hrem;
+};
+
+// The stencil's weights (negated: -c_k dt / dx) in both halves of a pair, as the packed
+// multiply-adds read them.
+struct ResStencil {
+    float2 nc[4];
+};
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{\n\t.reg .b64 a, b, r;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tsub.rn.f32x2 r, a, b;\n\t"
+        "mov.b64 {%0, %1}, r;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// c + s (a - b), both halves of s equal: ptap
+__device__ __forceinline__ float4 rtap(const float2 &s, const float4 &a, const float4 &b, const float4 &c)
+{
+    return cat4(__ffma2_rn(s, sub2(lo2(a), lo2(b)), lo2(c)), __ffma2_rn(s, sub2(hi2(a), hi2(b)), hi2(c)));
+}
+__device__ __forceinline__ float4 rscale(const float2 &s, const float4 &b)
+{
+    return cat4(__fmul2_rn(s, lo2(b)), __fmul2_rn(s, hi2(b)));
+}
+// row_dplus / row_dminus of a float4 b with the float4 a to its left and c to its right
+template <int M, bool PLUS>
+__device__ __forceinline__ float4 row_diff(const float4 &a, const float4 &b, const float4 &c, const float2 *cf)
+{
+    const float w[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+    float o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float g = 0.f;
+#pragma unroll
+        for (int k = 1; k <= M; ++k)
+            g = PLUS ? fmaf(cf[k - 1].x, w[4 + q + k] - w[4 + q - k + 1], g) : fmaf(cf[k - 1].x, w[4 + q + k - 1] - w[4 + q - k], g);
+        o[q] = g;
+    }
+    return make_float4(o[0], o[1], o[2], o[3]);
+}
+
+struct ResFwdArgs {
+    const float *p0, *vx0, *vz0;    // state before step n0 of shot 0 (null: zero)
+    float *p1, *vx1, *vz1;          // state after step n1 - 1 (null: not written)
+    float *hist;                    // p^{n0} .. p^{n1}, one slot a step (null: not kept)
+    long long slot;                 // floats between history slots
+    Model mo;
+    Dims d;
+    ResStencil st;
+    Source src;
+    const long long *ridx;          // receivers (traces non-null)
+    const float *rw;
+    float *traces;                  // [shots][nr][nt]
+    int nr, nt;
+    int n0, n1;
+    ResCut cut;
+    unsigned long long *mail;       // [shots][tiles][MAIL] mailboxes, cleared before the launch
+};
+
+// Four values and their step tag as two 16-byte stores; each 8-byte word is written whole.
+__device__ __forceinline__ void mail_put4(unsigned long long *m, const float4 &v, unsigned tag)
+{
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(m), "l"(t | __float_as_uint(v.x)),
+                 "l"(t | __float_as_uint(v.y))
+                 : "memory");
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(m + 2), "l"(t | __float_as_uint(v.z)),
+                 "l"(t | __float_as_uint(v.w))
+                 : "memory");
+}
+
+struct MailWord4 {
+    unsigned long long w[4];
+};
+
+__device__ __forceinline__ void mail_get4(const unsigned long long *m, MailWord4 &r)
+{
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(r.w[0]), "=l"(r.w[1]) : "l"(m) : "memory");
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(r.w[2]), "=l"(r.w[3]) : "l"(m + 2) : "memory");
+}
+
+__device__ __forceinline__ bool mail_ready(const MailWord4 &r, unsigned tag)
+{
+    return (unsigned)(r.w[0] >> 32) == tag && (unsigned)(r.w[1] >> 32) == tag && (unsigned)(r.w[2] >> 32) == tag &&
+           (unsigned)(r.w[3] >> 32) == tag;
+}
+
+__device__ __forceinline__ float4 mail_value(const MailWord4 &r)
+{
+    return make_float4(__uint_as_float((unsigned)r.w[0]), __uint_as_float((unsigned)r.w[1]),
+                       __uint_as_float((unsigned)r.w[2]), __uint_as_float((unsigned)r.w[3]));
+}
+
+// This CTA's tile.
+struct ResTile {
+    int t, s;            // tile of its shot, shot of the launch
+    int g0, ng;          // first column group, groups
+    int z0, h;           // first row, rows
+    bool L, R, U, D;     // has a neighbour
+};
+
+__device__ __forceinline__ ResTile res_tile(const ResCut &c, int block)
+{
+    ResTile T;
+    const int n = c.tx * c.tz;
+    T.s = block / n;
+    T.t = block - T.s * n;
+    const int tj = T.t / c.tx, ti = T.t - tj * c.tx;
+    T.g0 = ti * c.gbase + min(ti, c.grem);
+    T.ng = c.gbase + (ti < c.grem);
+    T.z0 = tj * c.hbase + min(tj, c.hrem);
+    T.h = c.hbase + (tj < c.hrem);
+    T.L = ti > 0;
+    T.R = ti + 1 < c.tx;
+    T.U = tj > 0;
+    T.D = tj + 1 < c.tz;
+    return T;
+}
+
+// Receivers of a tile (those whose first corner cell is its own).
+struct ResRec {
+    int n;               // receivers of the tile (above RES_RC every step scans them all)
+    int diag;            // a receiver reads the cell past the tile's lower right corner
+    int r[RES_RC], off[RES_RC];
+    float w[RES_RC][4];
+};
+
+// Shared memory of a forward CTA.
+template <class S>
+struct __align__(16) ResFwdSmem {
+    float p[S::E + S::HR][S::PP];            // row e at [e + HR]
+    float vz[S::E + 2 * S::M][S::PZ];        // row e at [e + 2M]
+    float2 az[S::E], azh[S::E];              // row e at [e + M], in both halves
+    int sj[4], si[4];                        // the shot's source cells relative to the tile
+    float sw[4];
+    ResRec rec;
+    int abort;                               // a wait of this CTA expired
+};
+
+// The tile's receivers (order irrelevant: each writes its own trace); offsets for pitch PP.
+__device__ __forceinline__ void res_receivers(ResRec &rc, const ResTile &T, const Dims &d, const long long *ridx,
+                                              const float *rw, int nr, int PP, int tid)
+{
+    for (int k = tid; k < nr; k += blockDim.x) {
+        const long long o = ridx[4 * k];
+        const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
+        if (j < 0 || j >= T.h || i < 0 || i >= 4 * T.ng) continue;
+        if (j == T.h - 1 && i == 4 * T.ng - 1) rc.diag = 1;
+        const int e = atomicAdd(&rc.n, 1);
+        if (e >= RES_RC) continue;
+        rc.r[e] = k;
+        rc.off[e] = j * PP + i;
+        for (int c = 0; c < 4; ++c) rc.w[e][c] = rw[4 * k + c];
+    }
+}
+
+// trace[s][r][n] of the tile's receivers from p^{n+1} (own cells and halo); `p`: own cell (0, 0)
+__device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, const Dims &d, const long long *ridx,
+                                           const float *rw, float *traces, int nr, int nt, int n, const float *p, int PP,
+                                           int tid)
+{
+    if (rc.n <= RES_RC) {
+        for (int k = tid; k < rc.n; k += blockDim.x) {
+            const float *q = p + rc.off[k];
+            float v = 0.f;
+            v += rc.w[k][0] * q[0];
+            v += rc.w[k][1] * q[1];
+            v += rc.w[k][2] * q[PP];
+            v += rc.w[k][3] * q[PP + 1];
+            traces[((long long)T.s * nr + rc.r[k]) * nt + n] = v;
+        }
+        return;
+    }
+    for (int k = tid; k < nr; k += blockDim.x) {
+        const long long o = ridx[4 * k];
+        const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
+        if (j < 0 || j >= T.h || i < 0 || i >= 4 * T.ng) continue;
+        const float *q = p + j * PP + i;
+        float v = 0.f;
+        v += rw[4 * k] * q[0];
+        v += rw[4 * k + 1] * q[1];
+        v += rw[4 * k + 2] * q[PP];
+        v += rw[4 * k + 3] * q[PP + 1];
+        traces[((long long)T.s * nr + k) * nt + n] = v;
+    }
+}
+
+// What a thread receives: the float4 tid, tid + nt, ... of the halo; the first two kept as
+// (mailbox word, offset from the field's own cell (0, 0)).
+template <class S>
+struct ResRecv {
+    int n, w0, o0, w1, o1;
+    __device__ ResRecv(const ResTile &T, int tid, int nt)
+    {
+        n = (T.U + T.D) * S::HR * T.ng + 2 * (T.L + T.R) * T.h;
+        item(T, tid, w0, o0);
+        item(T, tid + nt, w1, o1);
+    }
+    __device__ __forceinline__ void item(const ResTile &T, int k, int &word, int &off) const
+    {
+        const int nrow = S::HR * T.ng, nU = T.U ? nrow : 0, nD = T.D ? nrow : 0, nL = T.L ? 2 * T.h : 0;
+        if (k >= n) k = 0;
+        if (k < nU + nD) {
+            const bool up = k < nU;
+            const int q = up ? k : k - nU, r = q / T.ng, g = 4 * (q - r * T.ng);
+            word = (up ? 0 : S::MB) + r * S::W + g;
+            off = ((up ? -S::HR : T.h) + r) * S::PP + g;
+        } else {
+            k -= nU + nD;
+            const bool left = k < nL;
+            if (!left) k -= nL;
+            word = (left ? S::ML : S::MR) + 4 * k;
+            off = (k >> 1) * S::PP + (left ? -8 : 4 * T.ng) + 4 * (k & 1);
+        }
+    }
+    // words of step `tag` of this tile's mailbox slot m into the halo of the field whose own cell
+    // (0, 0) is at p; false when a wait expired
+    __device__ __forceinline__ bool get(const unsigned long long *m, const ResTile &T, float *p, unsigned tag, int tid,
+                                        int nt) const
+    {
+        int spin = 0;
+        if (tid < n) {
+            const bool two = tid + nt < n;
+            MailWord4 a, b;
+            mail_get4(m + w0, a);
+            if (two) mail_get4(m + w1, b);
+            while (!mail_ready(a, tag) && ++spin < RES_SPIN) mail_get4(m + w0, a);
+            st4(p + o0, mail_value(a));
+            if (two) {
+                while (!mail_ready(b, tag) && ++spin < RES_SPIN) mail_get4(m + w1, b);
+                st4(p + o1, mail_value(b));
+            }
+            for (int k = tid + 2 * nt; k < n; k += nt) {
+                int w, o;
+                item(T, k, w, o);
+                mail_get4(m + w, a);
+                while (!mail_ready(a, tag) && ++spin < RES_SPIN) mail_get4(m + w, a);
+                st4(p + o, mail_value(a));
+            }
+        }
+        return spin < RES_SPIN;
+    }
+};
+
+// What a lane sends of its own rows: up and down (rows within HR of the edge), and left or right
+// (the two groups at the edge; tiles with such a neighbour have at least 4 groups).
+template <class S>
+struct ResSend {
+    unsigned long long *ud, *lr;         // word of row 0 in the neighbour's slot; null: none
+    int dn;                              // down's offset from up
+    bool up, down;                       // this warp has rows for the neighbour
+    __device__ ResSend(unsigned long long *box, const ResTile &T, const ResCut &c, int g, int e0)
+    {
+        const bool own = g >= 0 && g < T.ng;
+        up = own && T.U && e0 < S::HR && e0 + S::R > 0;
+        down = own && T.D && e0 + S::R > T.h - S::HR && e0 < T.h;
+        ud = box - (long long)c.tx * S::MAIL + S::MB + 4 * g;
+        dn = 2 * c.tx * S::MAIL - S::MB - (T.h - S::HR) * S::W;
+        lr = own && T.L && g < 2 ? box - S::MAIL + S::MR + 4 * g
+             : own && T.R && g >= T.ng - 2 ? box + S::MAIL + S::ML + 4 * (g - (T.ng - 2)) : nullptr;
+    }
+    __device__ __forceinline__ void put(const ResTile &T, int slot, int e0, const float4 (&v)[S::R], unsigned tag) const
+    {
+        constexpr int R = S::R;
+        if (lr)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (e0 + r >= 0 && e0 + r < T.h) mail_put4(lr + slot + (e0 + r) * 8, v[r], tag);
+        if (up)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (e0 + r >= 0 && e0 + r < S::HR) mail_put4(ud + slot + (e0 + r) * S::W, v[r], tag);
+        if (down)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (e0 + r >= T.h - S::HR && e0 + r < T.h) mail_put4(ud + dn + slot + (e0 + r) * S::W, v[r], tag);
+    }
+};
+
+// The neighbours' float4 of a row held across the warp, those components an order-2M D- reads
+template <int M>
+__device__ __forceinline__ void warp_sides(const float4 &b, float4 &l, float4 &r)
+{
+    const unsigned all = 0xffffffffu;
+    l = r = f4(0.f);
+    if (M > 3) l.x = __shfl_up_sync(all, b.x, 1);
+    if (M > 2) l.y = __shfl_up_sync(all, b.y, 1);
+    l.z = __shfl_up_sync(all, b.z, 1);
+    l.w = __shfl_up_sync(all, b.w, 1);
+    r.x = __shfl_down_sync(all, b.x, 1);
+    if (M > 2) r.y = __shfl_down_sync(all, b.y, 1);
+    if (M > 3) r.z = __shfl_down_sync(all, b.z, 1);
+}
+
+// component i of v += kw * w, product and sum rounded apart (as the streaming kernels' injection)
+__device__ __forceinline__ void add_source(float4 &v, int i, float kw, float w)
+{
+    const float a = __fmul_rn(kw, w);
+    v.x = i == 0 ? __fadd_rn(v.x, a) : v.x;
+    v.y = i == 1 ? __fadd_rn(v.y, a) : v.y;
+    v.z = i == 2 ? __fadd_rn(v.z, a) : v.z;
+    v.w = i == 3 ? __fadd_rn(v.w, a) : v.w;
+}
+
+// Forward steps n0 .. n1 - 1.
+template <class S>
+__global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant__ ResFwdArgs a)
+{
+    constexpr int M = S::M, R = S::R, HR = S::HR, PP = S::PP, PZ = S::PZ;
+    extern __shared__ __align__(16) unsigned char fwi_smem[];
+    ResFwdSmem<S> &sh = *reinterpret_cast<ResFwdSmem<S> *>(fwi_smem);
+    const ResCut &c = a.cut;
+    const Dims &d = a.d;
+    const Model &mo = a.mo;
+    const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
+    const ResTile T = res_tile(c, blockIdx.x);
+    const long long so = (long long)T.s * d.Np;
+    int *stt = mo.status;
+
+    for (int k = tid; k < (int)(sizeof(ResFwdSmem<S>) / 4); k += nt) reinterpret_cast<int *>(fwi_smem)[k] = 0;
+    __syncthreads();
+    for (int k = tid; k < S::E; k += nt) {
+        const int j = T.z0 - M + k;
+        if (j >= 0 && j < d.Nz) {
+            sh.az[k] = make_float2(mo.az[j], mo.az[j]);
+            sh.azh[k] = make_float2(mo.azh[j], mo.azh[j]);
+        }
+    }
+    if (tid < 4) {
+        const long long o = a.src.idx[4 * T.s + tid];
+        sh.sj[tid] = (int)(o / d.Px) - T.z0;
+        sh.si[tid] = (int)(o % d.Px) - 4 * T.g0;
+        sh.sw[tid] = a.src.w[4 * T.s + tid];
+    }
+    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid);
+    float *const p00 = &sh.p[HR][8];                      // own cell (0, 0)
+    if (a.p0)   // initial pressure of the tile and its halo
+        for (int k = tid; k < (T.h + 2 * HR) * (T.ng + 4); k += nt) {
+            const int row = k / (T.ng + 4) - HR, g = k % (T.ng + 4) - 2;
+            const int j = T.z0 + row, i = 4 * (T.g0 + g);
+            const bool rin = row >= 0 && row < T.h, gin = g >= 0 && g < T.ng;
+            if (!rin && !gin) continue;                   // corners no stencil reads
+            if (FWI_IN(j >= 0 && j < d.Nz && i >= 0 && i < d.Nx, j * d.Px + i, 4, d.Np, stt))
+                st4(p00 + row * PP + 4 * g, ld4(a.p0 + so + j * d.Px + i));
+        }
+    __syncthreads();
+
+    // this lane's cells: group g, extended rows e0 .. e0 + R - 1
+    const int g = lane - 1, e0 = (tid >> 5) * R - M, col = 4 * (T.g0 + g);
+    const bool own = g >= 0 && g < T.ng, side = (g == -1 || g == T.ng) && col >= 0 && col < d.Nx;
+    const int go = (T.z0 + e0) * d.Px + col;
+    const float4 axv = ldg_if(mo.ax + col, own), axhv = ldg_if(mo.axh + col, own || side);
+    float4 p[R], vx[R], vz[R], Kv[R], bx[R], bz[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = e0 + r, j = T.z0 + e, o = go + r * d.Px;
+        const bool grid = j >= 0 && j < d.Nz, rin = e >= 0 && e < T.h, zin = e < T.h + M - 1;
+        const bool fx = FWI_IN(grid && rin && (own || side), o, 4, d.Np, stt), fz = FWI_IN(grid && zin && own, o, 4, d.Np, stt);
+        Kv[r] = ldg_if(mo.K + o, fz && rin);
+        bx[r] = ldg_if(mo.bx + o, fx);
+        bz[r] = ldg_if(mo.bz + o, fz);
+        p[r] = vx[r] = vz[r] = f4(0.f);
+        if (a.p0) {
+            if (fx) vx[r] = ld4(a.vx0 + so + o);
+            if (fz) vz[r] = ld4(a.vz0 + so + o);
+            p[r] = ld4(p00 + e * PP + 4 * g);   // own cells and halo; zero elsewhere
+        }
+        if (a.hist && fz && rin) st4(a.hist + so + o, p[r]);
+    }
+    bool hsrc = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        hsrc |= own && sh.si[k] >= 4 * g && sh.si[k] < 4 * g + 4 && sh.sj[k] >= max(e0, 0) && sh.sj[k] < min(e0 + R, T.h);
+    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * S::MAIL;
+    const ResSend<S> send(box, T, c, g, e0);
+    const ResRecv<S> recv(T, tid, nt);
+    float *const prow = p00 + e0 * PP + 4 * g;            // p of (e0, g)
+    float *const zrow = &sh.vz[e0 + 2 * M][4 * lane];     // v_z of (e0, g)
+    const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
+    float *hrow = a.hist ? a.hist + so + go : nullptr;
+    const float2 *const nc = a.st.nc;
+
+    const bool inner = e0 >= 0 && e0 + R <= T.h;          // every row of the warp is an own row
+    float wn = hsrc ? __ldg(a.src.wav + a.n0) : 0.f;
+    for (int n = a.n0; n < a.n1; ++n) {
+        // ---------------------------------------------------------------- velocities
+        {
+            float4 w[R + HR];   // p rows e0 - M + 1 .. e0 + R - 1 + M
+#pragma unroll
+            for (int q = 0; q < M - 1; ++q) w[q] = ld4(prow + (q - (M - 1)) * PP);
+#pragma unroll
+            for (int q = 0; q < R; ++q) w[M - 1 + q] = p[q];
+#pragma unroll
+            for (int q = 0; q < M; ++q) w[M - 1 + R + q] = ld4(prow + (R + q) * PP);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 gz = f4(0.f);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) gz = rtap(nc[k - 1], w[r + M - 1 + k], w[r + M - k], gz);
+                vz[r] = pmul(rscale(azhr[r], axv), pfma(bz[r], gz, vz[r]));
+                st4(zrow + r * PZ, vz[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 gx = row_diff<M, true>(ld4(prow + r * PP - 4), p[r], ld4(prow + r * PP + 4), nc);
+            vx[r] = pmul(rscale(azr[r], axhv), pfma(bx[r], gx, vx[r]));
+        }
+        __syncthreads();
+        // ------------------------------------------------------------------ pressure
+        const unsigned tag = (unsigned)(n - a.n0) + 1u;
+        const int slot = (n & 1) * S::SLOT;
+        if (hrow) hrow += a.slot;
+        {
+            float4 w[R + HR];   // v_z rows e0 - M .. e0 + R - 1 + M - 1
+#pragma unroll
+            for (int q = 0; q < M; ++q) w[q] = ld4(zrow + (q - M) * PZ);
+#pragma unroll
+            for (int q = 0; q < R; ++q) w[M + q] = vz[q];
+#pragma unroll
+            for (int q = 0; q < M - 1; ++q) w[M + R + q] = ld4(zrow + (R + q) * PZ);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 l, q;
+                warp_sides<M>(vx[r], l, q);
+                float4 dv = row_diff<M, false>(l, vx[r], q, nc);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) dv = rtap(nc[k - 1], w[r + M + k - 1], w[r + M - k], dv);
+                p[r] = pmul(rscale(azr[r], axv), pfma(Kv[r], dv, p[r]));
+            }
+            if (hsrc)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int e = e0 + r, i = sh.si[k] - 4 * g;
+                        if (sh.sj[k] == e && e >= 0 && e < T.h && i >= 0 && i < 4)
+                            add_source(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
+                    }
+            send.put(T, slot, e0, p, tag);
+            if (own) {
+                if (inner) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) st4(prow + r * PP, p[r]);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (e0 + r >= 0 && e0 + r < T.h) st4(prow + r * PP, p[r]);
+                }
+                if (hrow)
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (e0 + r >= 0 && e0 + r < T.h && FWI_IN(true, (long long)go + r * d.Px, 4, d.Np, stt))
+                            st4(hrow + r * d.Px, p[r]);
+            }
+            if (hsrc && n + 1 < a.n1) wn = __ldg(a.src.wav + n + 1);
+        }
+        // ------------------------------------------------------------------ exchange
+        if (e0 <= 0 && e0 + R > 0 && g == 0 && T.U && T.L) {   // the first cell, for the upper left diagonal tile
+            float v = 0.f;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (e0 + r == 0) v = p[r].x;
+            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(box - (long long)(c.tx + 1) * S::MAIL + 2 * S::SLOT + (n & 3)),
+                         "l"((unsigned long long)tag << 32 | __float_as_uint(v))
+                         : "memory");
+        }
+        bool ok = recv.get(box + slot, T, p00, tag, tid, nt);
+        if (tid == 0 && sh.rec.diag && T.R && T.D) {
+            unsigned long long v = 0;
+            int spin = 0;
+            do {
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(box + 2 * S::SLOT + (n & 3)) : "memory");
+            } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
+            ok = ok && spin < RES_SPIN;
+            p00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
+        }
+        if (!ok) {
+            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
+            atomicOr(stt, ST_ETIMEOUT);
+        }
+        __syncthreads();
+        if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
+        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, p00, PP, tid);
+        // the halo's pressure: the groups beside the tile, and the rows above and below it
+        if (!own || !inner)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (!own || e0 + r < 0 || e0 + r >= T.h) p[r] = ld4(prow + r * PP);
+    }
+    if (a.p1)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int e = e0 + r, o = go + r * d.Px;
+            if (FWI_IN(own && e >= 0 && e < T.h, o, 4, d.Np, stt)) {
+                st4(a.p1 + so + o, p[r]);
+                st4(a.vx1 + so + o, vx[r]);
+                st4(a.vz1 + so + o, vz[r]);
+            }
+        }
+}
+
+}  // namespace fwi
