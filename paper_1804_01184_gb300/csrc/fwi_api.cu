@@ -685,7 +685,7 @@ int forward_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const size_t bf = (size_t)bg * P.d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * P.d.Np;   // floats between snapshot slots
     ResPlan rp;
-    if (res_wanted(P, bg, rp)) {
+    if (res_wanted(P, RES_FWD, bg, rp)) {
         const int C = with_hist ? P.C : P.nt;
         for (int n0 = 0; n0 < P.nt; n0 += C) {
             const int n1 = std::min(n0 + C, P.nt);
@@ -752,7 +752,9 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const Fwd f{P, work, st, wav};
     const size_t bf = (size_t)bg * d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * d.Np;
-    const int first = P.nt & 1;   // buffers holding pbar^{nt}, vbar^{nt-1/2} = 0
+    ResPlan ra;
+    const bool chip = res_wanted(P, RES_ADJ, bg, ra);
+    int first = P.nt & 1;         // buffers holding pbar^{nt}, vbar^{nt-1/2} = 0
     CK(cudaMemsetAsync(at<char>(work, P.ap[first]), 0, bf, st));
     CK(cudaMemsetAsync(at<char>(work, P.avx[first]), 0, bf, st));
     CK(cudaMemsetAsync(at<char>(work, P.avz[first]), 0, bf, st));
@@ -762,7 +764,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
         if (k < P.nseg - 1) {   // recompute the segment from its checkpoint
             TraceRange tr(PH_RECOMPUTE);
             ResPlan rp;
-            if (res_wanted(P, bg, rp)) {
+            if (res_wanted(P, RES_FWD, bg, rp)) {
                 const int rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, k), ResState{}, snap,
                                            nullptr);
                 if (rc) return rc;
@@ -776,7 +778,21 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
             }
         }
         TraceRange tr(PH_ADJOINT);
-        for (int n = n1 - 1; n >= n0; --n) {
+        // on chip: launches that end where an accumulation chunk or the segment does
+        for (int n = n1 - 1; chip && n >= n0;) {
+            const int lo = std::max(n / P.acc * P.acc, n0);
+            const float *pl = snap + (size_t)(lo - n0) * slot;
+            if (P.nr > 0)
+                LAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[first]),
+                       at<float>(work, P.accK), snap + (size_t)(n + 1 - n0) * slot, bg, P.nr, P.nt, n, d.Np,
+                       at<long long>(work, P.ridx), at<float>(work, P.rw), at<int>(work, P.rl), res);
+            int rc = res_adjoint(P, work, st, ra, bg, n, lo, first, pl, res);
+            if (rc) return rc;
+            first ^= 1;
+            if (lo % P.acc == 0 && (rc = flush_acc(P, work, bg, st))) return rc;
+            n = lo - 1;
+        }
+        for (int n = n1 - 1; !chip && n >= n0; --n) {
             const float *pn = snap + (size_t)(n - n0) * slot, *pn1 = snap + (size_t)(n + 1 - n0) * slot;
             if (P.nr > 0)   // pbar^{n+1} += R^T r_n, with its K-gradient term (R^T r_n) p^{n+1}
                 LAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[(n + 1) & 1]),

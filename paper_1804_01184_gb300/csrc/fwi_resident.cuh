@@ -561,4 +561,307 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
         }
 }
 
+// ------------------------------------------------------------- adjoint steps (S7)
+//
+// Reverse steps nhi, nhi - 1, .. nlo of the adjoint scheme (see fwi_warp.cuh) with the gradient
+// products, kept on chip like the forward steps.  The exchanged field is q = K d_p pbar, which is
+// all the stencils read of pbar beyond a tile.  The accumulators and the step's forward pressure
+// (copied in one step ahead by cp.async) sit in shared memory.  The receivers' residual of the
+// next step is added to pbar, with its K-gradient term, before q is formed; the caller has added
+// step nhi's.
+
+constexpr int RES_ENT = 256;    // injection cells of a tile listed in shared memory
+using ResAdj2 = ResShape<2, 4, 12>;
+using ResAdj4 = ResShape<4, 4, 12>;
+
+struct ResAdjArgs {
+    const float *ap0, *avx0, *avz0;   // pbar^{nhi+1} (injected), vbar of the launch's shots
+    float *ap1, *avx1, *avz1;         // pbar^{nlo}, vbar after step nlo (other buffers)
+    const float *pn;                  // p^{nlo}, one slot a step
+    long long slot;
+    float *accK, *accBx, *accBz;      // FP32 accumulators, read and written once
+    Model mo;
+    Dims d;
+    ResStencil st;                    // c_k dt / dx (not negated)
+    const long long *ridx;
+    const float *rw;
+    const int *rl;                    // chains of footprint entries that share a cell
+    const float *res;                 // [shots][nr][nt]
+    int nr, nt;
+    int nhi, nlo;
+    ResCut cut;
+    unsigned long long *mail;
+};
+
+template <class S>
+struct __align__(16) ResAdjSmem {
+    float q[S::E + S::HR][S::PP];            // row e at [e + HR], column c at [c + 8]
+    float pn[2][S::E + S::HR][S::PP];        // forward pressure of this step and the next
+    float bz[S::E + 2 * S::M][S::PZ];        // b_z u_z: row e at [e + 2M]
+    float acc[3][S::E][128];                 // K, b_x, b_z: row e at [e + M], lane l at 4 l
+    float inj[S::E][128];                    // the next step's injection, zero off the receivers
+    float2 az[S::E], azh[S::E];              // row e at [e + M], in both halves
+    int cell[RES_ENT], ent[RES_ENT];         // injection cells: offset in inj, first footprint entry
+    int has[S::E];                           // the row holds an injection cell
+    int nent;
+    int abort;
+};
+
+// acc + v as the streaming kernels' red.global.add.f32 adds it: subnormals flush to zero
+__device__ __forceinline__ float4 add_ftz(const float4 &a, const float4 &v)
+{
+    float4 r;
+    asm("add.rn.ftz.f32 %0, %1, %2;" : "=f"(r.x) : "f"(a.x), "f"(v.x));
+    asm("add.rn.ftz.f32 %0, %1, %2;" : "=f"(r.y) : "f"(a.y), "f"(v.y));
+    asm("add.rn.ftz.f32 %0, %1, %2;" : "=f"(r.z) : "f"(a.z), "f"(v.z));
+    asm("add.rn.ftz.f32 %0, %1, %2;" : "=f"(r.w) : "f"(a.w), "f"(v.w));
+    return r;
+}
+
+template <class S>
+__global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant__ ResAdjArgs a)
+{
+    constexpr int M = S::M, R = S::R, HR = S::HR, PP = S::PP, PZ = S::PZ;
+    extern __shared__ __align__(16) unsigned char fwi_smem[];
+    ResAdjSmem<S> &sh = *reinterpret_cast<ResAdjSmem<S> *>(fwi_smem);
+    const ResCut &c = a.cut;
+    const Dims &d = a.d;
+    const Model &mo = a.mo;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+    const ResTile T = res_tile(c, blockIdx.x);
+    const long long so = (long long)T.s * d.Np;
+    int *stt = mo.status;
+
+    for (int k = tid; k < (int)(sizeof(ResAdjSmem<S>) / 4); k += nt) reinterpret_cast<int *>(fwi_smem)[k] = 0;
+    __syncthreads();
+    for (int k = tid; k < S::E; k += nt) {
+        const int j = T.z0 - M + k;
+        if (j >= 0 && j < d.Nz) {
+            sh.az[k] = make_float2(mo.az[j], mo.az[j]);
+            sh.azh[k] = make_float2(mo.azh[j], mo.azh[j]);
+        }
+    }
+    // the cell of footprint entry k in inj, -1 when another entry leads its chain or it is not here
+    auto entry_cell = [&](int k) {
+        if (!(a.rl[k] & CHAIN_FIRST)) return -1;
+        const long long o = a.ridx[k];
+        const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
+        return j >= 0 && j < T.h && i >= 0 && i < 4 * T.ng ? (j + M) * 128 + 4 + i : -1;
+    };
+    for (int k = tid; k < 4 * a.nr; k += nt) {
+        const int o = entry_cell(k);
+        if (o < 0) continue;
+        sh.has[o >> 7] = 1;
+        const int e = atomicAdd(&sh.nent, 1);
+        if (e < RES_ENT) {
+            sh.cell[e] = o;
+            sh.ent[e] = k;
+        }
+    }
+    float *const q00 = &sh.q[HR][8], *const p00 = &sh.pn[0][HR][8];   // own cell (0, 0)
+    constexpr int PB = (S::E + HR) * PP;                              // floats of a pn buffer
+    // q of the tile and its halo
+    for (int k = tid; k < (T.h + 2 * HR) * (T.ng + 4); k += nt) {
+        const int row = k / (T.ng + 4) - HR, g = k % (T.ng + 4) - 2;
+        const int j = T.z0 + row, i = 4 * (T.g0 + g), o = j * d.Px + i;
+        const bool rin = row >= 0 && row < T.h, gin = g >= 0 && g < T.ng;
+        if (!rin && !gin) continue;                   // corners no stencil reads
+        if (FWI_IN(j >= 0 && j < d.Nz && i >= 0 && i < d.Nx, o, 4, d.Np, stt))
+            st4(q00 + row * PP + 4 * g, pmul(pmul(mo.az[j], ldg4(mo.ax + i)), pmul(ldg4(mo.K + o), ld4(a.ap0 + so + o))));
+    }
+    // forward pressure of step n: rows -(M - 1) .. h + M - 1, the tile's groups and one beside each
+    auto fetch = [&](int n, int buf) {
+        const float *src = a.pn + (long long)(n - a.nlo) * a.slot + so;
+        const int gl = lane - 1, i = 4 * (T.g0 + gl);
+        const bool ok = gl <= T.ng && i >= 0 && i < d.Nx;
+        for (int row = warp - (M - 1); row < T.h + M; row += nw) {
+            const int j = T.z0 + row;
+            if (FWI_IN(ok && j >= 0 && j < d.Nz, j * d.Px + i, 4, d.Np, stt))
+                cp16(p00 + buf * PB + row * PP + 4 * gl, src, j * d.Px + i, true);
+        }
+        cp_commit();
+    };
+    fetch(a.nhi, 0);
+
+    // this lane's cells: group g, extended rows e0 .. e0 + R - 1
+    const int g = lane - 1, e0 = warp * R - M, col = 4 * (T.g0 + g);
+    const bool own = g >= 0 && g < T.ng, side = (g == -1 || g == T.ng) && col >= 0 && col < d.Nx;
+    const int go = (T.z0 + e0) * d.Px + col;
+    const float4 axv = ldg_if(mo.ax + col, own), axhv = ldg_if(mo.axh + col, own || side);
+    float4 pb[R], ux[R], uz[R], Kv[R], bx[R], bz[R];
+    float *const acck = &sh.acc[0][e0 + M][4 * lane], *const accx = &sh.acc[1][e0 + M][4 * lane],
+                *const accz = &sh.acc[2][e0 + M][4 * lane];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = e0 + r, j = T.z0 + e, o = go + r * d.Px;
+        const bool grid = j >= 0 && j < d.Nz, rin = e >= 0 && e < T.h, zin = e < T.h + M - 1;
+        const bool fx = FWI_IN(grid && rin && (own || side), o, 4, d.Np, stt), fz = FWI_IN(grid && zin && own, o, 4, d.Np, stt);
+        Kv[r] = ldg_if(mo.K + o, fz && rin);
+        bx[r] = ldg_if(mo.bx + o, fx);
+        bz[r] = ldg_if(mo.bz + o, fz);
+        pb[r] = ux[r] = uz[r] = f4(0.f);
+        if (fx) ux[r] = ld4(a.avx0 + so + o);
+        if (fz) uz[r] = ld4(a.avz0 + so + o);
+        if (fz && rin) {
+            pb[r] = ld4(a.ap0 + so + o);
+            st4(acck + r * 128, ld4(a.accK + so + o));
+            st4(accx + r * 128, ld4(a.accBx + so + o));
+            st4(accz + r * 128, ld4(a.accBz + so + o));
+        }
+    }
+    __syncthreads();
+    unsigned hinj = 0;                                    // this warp's rows with injection cells
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (own && sh.has[e0 + r + M]) hinj |= 1u << r;
+    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * S::MAIL;
+    const ResSend<S> send(box, T, c, g, e0);
+    const ResRecv<S> recv(T, tid, nt);
+    float *const qrow = q00 + e0 * PP + 4 * g;
+    const float *const prow = p00 + e0 * PP + 4 * g;
+    float *const zrow = &sh.bz[e0 + 2 * M][4 * lane];
+    const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
+    const float2 *const cf = a.st.nc;
+    const bool inner = e0 >= 0 && e0 + R <= T.h;
+    const float *const rs = a.res + (long long)T.s * a.nr * a.nt;
+    const int n4 = 4 * a.nr, nent = sh.nent;
+    // this thread's first listed cell: its leading residual, loaded a step ahead
+    const bool lead = nent <= RES_ENT && tid < nent;
+    const int ek = lead ? sh.ent[tid] : 0, eo = lead ? sh.cell[tid] : 0;
+    float rv = lead && a.nhi > a.nlo ? rs[(long long)(ek >> 2) * a.nt + a.nhi - 1] : 0.f;
+    // sum over the chain of entry k of its residuals at step n, the leading one given
+    auto chain = [&](int k, int n, float first) {
+        float v = __fmul_rn(a.rw[k], first);
+        for (int m = a.rl[k] & (CHAIN_FIRST - 1); m < n4; m = a.rl[m] & (CHAIN_FIRST - 1))
+            v = fmaf(a.rw[m], rs[(long long)(m >> 2) * a.nt + n], v);
+        return v;
+    };
+    cp_wait<0>();
+    __syncthreads();
+
+    for (int n = a.nhi; n >= a.nlo; --n) {
+        const int it = a.nhi - n, buf = it & 1;
+        const float *const pr = prow + buf * PB;
+        if (n > a.nlo) fetch(n - 1, buf ^ 1);
+        else cp_commit();
+        // the injection of step n - 1 (added below, after pbar^n)
+        if (n > a.nlo) {
+            if (nent <= RES_ENT) {
+                if (lead) {
+                    (&sh.inj[0][0])[eo] = chain(ek, n - 1, rv);
+                    if (n - 1 > a.nlo) rv = rs[(long long)(ek >> 2) * a.nt + n - 2];
+                }
+                for (int k = tid + nt; k < nent; k += nt) {
+                    const int e = sh.ent[k];
+                    (&sh.inj[0][0])[sh.cell[k]] = chain(e, n - 1, rs[(long long)(e >> 2) * a.nt + n - 1]);
+                }
+            } else {
+                for (int k = tid; k < n4; k += nt) {
+                    const int o = entry_cell(k);
+                    if (o >= 0) (&sh.inj[0][0])[o] = chain(k, n - 1, rs[(long long)(k >> 2) * a.nt + n - 1]);
+                }
+            }
+        }
+        // ---------------------------------------------------------------- velocities
+        {
+            float4 w[R + HR];   // q rows e0 - M + 1 .. e0 + R - 1 + M
+#pragma unroll
+            for (int k = 0; k < R + HR; ++k) w[k] = ld4(qrow + (k - (M - 1)) * PP);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 gq = f4(0.f);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) gq = rtap(cf[k - 1], w[r + M - 1 + k], w[r + M - k], gq);
+                uz[r] = pmul(rscale(azhr[r], axv), padd(uz[r], gq));
+                st4(zrow + r * PZ, pmul(bz[r], uz[r]));
+                const float4 gx = row_diff<M, true>(ld4(qrow + r * PP - 4), w[r + M - 1], ld4(qrow + r * PP + 4), cf);
+                ux[r] = pmul(rscale(azr[r], axhv), padd(ux[r], gx));
+            }
+        }
+        {
+            float4 w[R + HR];   // p^n rows
+#pragma unroll
+            for (int k = 0; k < R + HR; ++k) w[k] = ld4(pr + (k - (M - 1)) * PP);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 gp = f4(0.f);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) gp = rtap(cf[k - 1], w[r + M - 1 + k], w[r + M - k], gp);
+                st4(accz + r * 128, add_ftz(ld4(accz + r * 128), pmul(uz[r], gp)));
+                const float4 gx = row_diff<M, true>(ld4(pr + r * PP - 4), w[r + M - 1], ld4(pr + r * PP + 4), cf);
+                st4(accx + r * 128, add_ftz(ld4(accx + r * 128), pmul(ux[r], gx)));
+            }
+        }
+        __syncthreads();
+        // ------------------------------------------------------------------ pressure
+        const unsigned tag = (unsigned)it + 1u;
+        const int slot = (it & 1) * S::SLOT;
+        {
+            float4 w[R + HR];   // b_z u_z rows e0 - M .. e0 + R - 1 + M - 1
+#pragma unroll
+            for (int k = 0; k < M; ++k) w[k] = ld4(zrow + (k - M) * PZ);
+#pragma unroll
+            for (int k = 0; k < R; ++k) w[M + k] = pmul(bz[k], uz[k]);
+#pragma unroll
+            for (int k = 0; k < M - 1; ++k) w[M + R + k] = ld4(zrow + (R + k) * PZ);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float4 bu = pmul(bx[r], ux[r]);
+                float4 l, rr;
+                warp_sides<M>(bu, l, rr);
+                float4 dv = row_diff<M, false>(l, bu, rr, cf);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) dv = rtap(cf[k - 1], w[r + M + k - 1], w[r + M - k], dv);
+                pb[r] = pfma(rscale(azr[r], axv), pb[r], dv);
+                st4(acck + r * 128, add_ftz(ld4(acck + r * 128), pmul(ld4(pr + r * PP), dv)));
+            }
+        }
+        if (n == a.nlo) break;
+        if (hinj) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (hinj >> r & 1) {
+                    const float4 v = ld4(&sh.inj[e0 + r + M][4 * lane]), p = ld4(pr + r * PP);
+                    float4 k = ld4(acck + r * 128);
+                    if (v.x != 0.f) { pb[r].x = __fadd_rn(pb[r].x, v.x); k.x = fmaf(v.x, p.x, k.x); }
+                    if (v.y != 0.f) { pb[r].y = __fadd_rn(pb[r].y, v.y); k.y = fmaf(v.y, p.y, k.y); }
+                    if (v.z != 0.f) { pb[r].z = __fadd_rn(pb[r].z, v.z); k.z = fmaf(v.z, p.z, k.z); }
+                    if (v.w != 0.f) { pb[r].w = __fadd_rn(pb[r].w, v.w); k.w = fmaf(v.w, p.w, k.w); }
+                    st4(acck + r * 128, k);
+                }
+        }
+        // ------------------------------------------------------------------ exchange
+        {
+            float4 q[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) q[r] = pmul(rscale(azr[r], axv), pmul(Kv[r], pb[r]));
+            send.put(T, slot, e0, q, tag);
+            if (own)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (inner || (e0 + r >= 0 && e0 + r < T.h)) st4(qrow + r * PP, q[r]);
+        }
+        if (!recv.get(box + slot, T, q00, tag, tid, nt)) {
+            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
+            atomicOr(stt, ST_ETIMEOUT);
+        }
+        cp_wait<0>();
+        __syncthreads();
+        if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
+    }
+    cp_wait<0>();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = e0 + r, o = go + r * d.Px;
+        if (FWI_IN(own && e >= 0 && e < T.h, o, 4, d.Np, stt)) {
+            st4(a.ap1 + so + o, pb[r]);
+            st4(a.avx1 + so + o, ux[r]);
+            st4(a.avz1 + so + o, uz[r]);
+            st4(a.accK + so + o, ld4(acck + r * 128));
+            st4(a.accBx + so + o, ld4(accx + r * 128));
+            st4(a.accBz + so + o, ld4(accz + r * 128));
+        }
+    }
+}
+
 }  // namespace fwi

@@ -105,6 +105,20 @@ def test_gradient_history_and_checkpoints(F, every):
     assert torch.equal(ref[0], got[0]) and torch.equal(ref[1], got[1])
 
 
+@pytest.mark.parametrize("nx,nz,order,sponge", GRIDS)
+def test_adjoint_is_bitwise_the_streaming_kernels(F, nx, nz, order, sponge):
+    """Two accumulation chunks, receivers that share cells and more of them than a tile lists."""
+    w = case(nx, nz, order, sponge, nt=70)
+    hi = np.array([(nx - 1) * w.dx, (nz - 1) * w.dx])
+    more = (hi * np.random.default_rng(3).random((90, 2))).astype(np.float32)
+    w.rec_xy = np.concatenate([w.rec_xy, more, more[::5]]).astype(np.float32)
+    g = gpu_grid(w)
+    res = I.random_like((w.ns, len(w.rec_xy), w.nt), 11, 1.0)
+    ref, got = both(F, lambda: F.fwi_adjoint(g, w.pz, w.xi_a, w.xi_b, w.src_xy, w.wavelet, w.rec_xy, res), "k_res_adj")
+    assert ref.abs().max().item() > 0
+    assert torch.equal(ref, got)
+
+
 def test_more_shots_than_a_launch_holds(F):
     w = case(201, 201, 8, 40, ns=33, nr=20, nt=30)
     g = gpu_grid(w)
