@@ -324,20 +324,15 @@ int setup(const Plan &P, const fwi_grid *g, int pz, const float *xa, const float
            at<float>(work, P.bx), at<float>(work, P.bz), status);
     const double sv = g->sponge_v > 0 ? g->sponge_v : g->vp_o;
     const double sR = (g->sponge_R > 0 && g->sponge_R < 1) ? g->sponge_R : 1e-3;
-    LAUNCH(fwi::k_sponge, (d.Px + 127) / 128, 128, 0, st, at<float>(work, P.ax), d.Px, d.nx, d.S, g->dx, g->dt, sv, sR, 0);
-    LAUNCH(fwi::k_sponge, (d.Px + 127) / 128, 128, 0, st, at<float>(work, P.axh), d.Px, d.nx, d.S, g->dx, g->dt, sv, sR, 1);
-    LAUNCH(fwi::k_sponge, (d.Nz + 127) / 128, 128, 0, st, at<float>(work, P.az), d.Nz, d.nz, d.S, g->dx, g->dt, sv, sR, 0);
-    LAUNCH(fwi::k_sponge, (d.Nz + 127) / 128, 128, 0, st, at<float>(work, P.azh), d.Nz, d.nz, d.S, g->dx, g->dt, sv, sR, 1);
-    if (src->ns > 0)
-        LAUNCH(fwi::k_geometry, (src->ns + 127) / 128, 128, 0, st, src->xy, src->ns, d, g->dx,
-               g->dt / (g->dx * g->dx), at<long long>(work, P.sidx), at<float>(work, P.sw), status);
-    if (rec->nr > 0) {
-        LAUNCH(fwi::k_geometry, (rec->nr + 127) / 128, 128, 0, st, rec->xy, rec->nr, d, g->dx, 1.0,
-               at<long long>(work, P.ridx), at<float>(work, P.rw), status);
-        if (adjoint)   // only injection reads the chains
-            LAUNCH(fwi::k_receiver_chain, (4 * rec->nr + 127) / 128, 128, 0, st, at<long long>(work, P.ridx), 4 * rec->nr,
-                   at<int>(work, P.rl));
-    }
+    const fwi::SetupArgs sa{d, g->dx, g->dt, sv, sR, g->dt / (g->dx * g->dx), at<float>(work, P.ax), at<float>(work, P.axh),
+                            at<float>(work, P.az), at<float>(work, P.azh), src->ns, rec->nr, src->xy, rec->xy,
+                            at<long long>(work, P.sidx), at<long long>(work, P.ridx), at<float>(work, P.sw),
+                            at<float>(work, P.rw), status};
+    const long long entries = 2LL * (d.Px + d.Nz) + src->ns + rec->nr;
+    LAUNCH(fwi::k_setup, (unsigned)((entries + 63) / 64), 64, 0, st, sa);
+    if (adjoint && rec->nr > 0)   // only injection reads the chains
+        LAUNCH(fwi::k_receiver_chain, (4 * rec->nr + fwi::CHAIN_NT - 1) / fwi::CHAIN_NT, fwi::CHAIN_NT, 0, st,
+               at<long long>(work, P.ridx), 4 * rec->nr, at<int>(work, P.rl));
     return FWI_OK;
 }
 
@@ -843,11 +838,12 @@ int finalize_grad(const Plan &P, const fwi_grid *g, int pz, const float *xa, con
 {
     TraceRange tr(PH_REDUCE);
     const fwi::Dims &d = P.d;
-    dim3 b2(32, 8), gp((d.Nx + 31) / 32, (d.Nz + 7) / 8), gq((d.nx + 31) / 32, (d.nz + 7) / 8);
-    LAUNCH(fwi::k_grad_cells, gp, b2, 0, st, at<float>(work, P.K), at<float>(work, P.bx), at<float>(work, P.bz), d,
-           at<double>(work, P.gK), at<double>(work, P.hx), at<double>(work, P.hz));
-    LAUNCH(fwi::k_grad_final, gq, b2, 0, st, at<double>(work, P.gK), at<double>(work, P.hx),
-           at<double>(work, P.hz), xa, xb, pz, g->vp_o, g->rho_o, d, grads);
+    // the folded rows take the adjoint fields' place (24 bytes a padded cell, 16 a row entry needed)
+    double *fold = at<double>(work, P.ap[0]);
+    LAUNCH(fwi::k_grad_fold, d.Nz, fwi::FOLD_NT, 0, st, at<float>(work, P.K), at<float>(work, P.bx), at<float>(work, P.bz), d,
+           at<double>(work, P.gK), at<double>(work, P.hx), at<double>(work, P.hz), fold);
+    dim3 b2(32, 8), gq((d.nx + 31) / 32, (d.nz + 7) / 8);
+    LAUNCH(fwi::k_grad_final, gq, b2, 0, st, fold, xa, xb, pz, g->vp_o, g->rho_o, d, grads);
     return FWI_OK;
 }
 

@@ -76,30 +76,46 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? l
 
 // K, bx = 2/(rho_i + rho_{i+1}), bz likewise, on the padded grid (padding copies the
 // nearest physical cell; the last node reuses its own rho).  Checks 1 + xi > 0 and the
-// CFL bound dt vp sqrt(2) sum|c_k| / dx <= 1.
-__global__ void k_model(const float *__restrict__ xa, const float *__restrict__ xb, int pz,
-                        double vp_o, double rho_o, double cfl_coef, Dims d,
-                        float *__restrict__ K, float *__restrict__ bx, float *__restrict__ bz,
-                        int *status)
+// CFL bound dt vp sqrt(2) sum|c_k| / dx <= 1.  The FP64 maps bound it, so a block evaluates
+// each of its cells and the row and column beside it once (not three times a cell: 61 -> 47 us
+// at 681 x 681, with the squared CFL test).  Blocks of 32 x 8 threads.
+__global__ void __launch_bounds__(256) k_model(const float *__restrict__ xa, const float *__restrict__ xb, int pz,
+                                               double vp_o, double rho_o, double cfl_coef, Dims d,
+                                               float *__restrict__ K, float *__restrict__ bx, float *__restrict__ bz,
+                                               int *status)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+    __shared__ double sr[9][33];
+    __shared__ bool sok[9][33];
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 8, tx = threadIdx.x, ty = threadIdx.y;
+    const int i = i0 + tx, j = j0 + ty;
+    double Kc = 0.0;
+    for (int k = ty * 32 + tx; k < 9 * 33; k += 256) {
+        // the block's own cells first (thread k's own cell is entry k), then the column and the row
+        const int c = k < 256 ? k % 32 : k < 265 ? 32 : k - 265, r = k < 256 ? k / 32 : k < 265 ? k - 256 : 8;
+        const int ii = min(i0 + c, d.Nx - 1), jj = min(j0 + r, d.Nz - 1);
+        const int pi = clampi(ii - d.S, 0, d.nx - 1), pj = clampi(jj - d.S, 0, d.nz - 1);
+        const long long q = (long long)pj * d.nx + pi;
+        double Kv = 0.0, rv = 0.0;
+        sok[r][c] = kr_of(pz, xa[q], xb[q], vp_o, rho_o, Kv, rv);
+        sr[r][c] = rv;
+        if (k < 256) Kc = Kv;
+    }
+    __syncthreads();
     if (i >= d.Px || j >= d.Nz) return;
     const long long o = cell(d, i, j);
     if (i >= d.Nx) { K[o] = 0.f; bx[o] = 0.f; bz[o] = 0.f; return; }
-    auto phys = [&](int ii, int jj, double &Kv, double &rv) {
-        int pi = clampi(ii - d.S, 0, d.nx - 1), pj = clampi(jj - d.S, 0, d.nz - 1);
-        long long q = (long long)pj * d.nx + pi;
-        return kr_of(pz, xa[q], xb[q], vp_o, rho_o, Kv, rv);
-    };
-    double Kc, rc, Kx, rx, Kz, rz;
-    bool ok = phys(i, j, Kc, rc);
-    ok = phys(i + 1 < d.Nx ? i + 1 : i, j, Kx, rx) && ok;
-    ok = phys(i, j + 1 < d.Nz ? j + 1 : j, Kz, rz) && ok;
-    if (!ok) { atomicOr(status, ST_EINVAL); K[o] = 0.f; bx[o] = 0.f; bz[o] = 0.f; return; }
-    if (sqrt(Kc / rc) * cfl_coef > 1.0) atomicOr(status, ST_ECFL);
+    // beyond the last node its own values stand (clamped above)
+    if (!(sok[ty][tx] && sok[ty][tx + 1] && sok[ty + 1][tx])) {
+        atomicOr(status, ST_EINVAL);
+        K[o] = 0.f; bx[o] = 0.f; bz[o] = 0.f;
+        return;
+    }
+    const double rc = sr[ty][tx];
+    // the squared form, clear of rounding, spares most cells the FP64 quotient and root
+    if (!(Kc * (cfl_coef * cfl_coef) < rc * (1.0 - 1e-9)) && sqrt(Kc / rc) * cfl_coef > 1.0) atomicOr(status, ST_ECFL);
     K[o] = (float)Kc;
-    bx[o] = (float)(2.0 / (rc + rx));
-    bz[o] = (float)(2.0 / (rc + rz));
+    bx[o] = (float)(2.0 / (rc + sr[ty][tx + 1]));
+    bz[o] = (float)(2.0 / (rc + sr[ty + 1][tx]));
 }
 
 // Born perturbation of the model: dK = J dxi, drho likewise (Jacobian of the map above),
@@ -151,11 +167,9 @@ __global__ void k_model_pert(const float *__restrict__ xa, const float *__restri
 
 // Sponge profile along one axis: n physical nodes, S cells each side; half = 1 for the
 // half nodes.  sigma = sigma_max (delta/S)^2, sigma_max = 3 v ln(1/R) / (2 S dx), d = exp(-sigma dt).
-__global__ void k_sponge(float *__restrict__ out, int len, int n, int S, double dx, double dt,
-                         double v, double R, int half)
+__device__ __forceinline__ void sponge_entry(float *__restrict__ out, int i, int n, int S, double dx, double dt,
+                                             double v, double R, int half)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= len) return;
     const int N = n + 2 * S;
     if (i >= N) { out[i] = 0.f; return; }
     const double u = i + (half ? 0.5 : 0.0);
@@ -170,11 +184,9 @@ __global__ void k_sponge(float *__restrict__ out, int len, int n, int S, double 
 
 // Bilinear footprint of point k: four (cell offset, weight * scale) pairs.  A point on the
 // last node puts its weight on (i0 + 1).  Points outside the physical grid flag EINVAL.
-__global__ void k_geometry(const float *__restrict__ xy, int n, Dims d, double dx, double scale,
-                           long long *__restrict__ idx, float *__restrict__ w, int *status)
+__device__ __forceinline__ void footprint_entry(const float *__restrict__ xy, int k, const Dims &d, double dx, double scale,
+                                                long long *__restrict__ idx, float *__restrict__ w, int *status)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
     const double x = xy[2 * k], z = xy[2 * k + 1];
     if (!(x >= 0.0 && z >= 0.0 && x <= (d.nx - 1) * dx && z <= (d.nz - 1) * dx)) {
         atomicOr(status, ST_EINVAL);
@@ -192,22 +204,70 @@ __global__ void k_geometry(const float *__restrict__ xy, int n, Dims d, double d
     idx[4 * k + 3] = cell(d, i0 + 1, j0 + 1);  w[4 * k + 3] = (float)(scale * tx * tz);
 }
 
+// The sponge profiles and the footprints of an operation in one launch (six launches of a few
+// hundred FP64 threads each cost 47 us).  One thread an entry: ax, axh (Px each), az, azh (Nz
+// each), sources, receivers.
+struct SetupArgs {
+    Dims d;
+    double dx, dt, sv, sR, src_scale;
+    float *ax, *axh, *az, *azh;
+    int ns, nr;
+    const float *src_xy, *rec_xy;
+    long long *sidx, *ridx;
+    float *sw, *rw;
+    int *status;
+};
+
+__global__ void __launch_bounds__(64) k_setup(SetupArgs a)
+{
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const Dims &d = a.d;
+    if (k < 2 * d.Px) {
+        const int half = k >= d.Px;
+        sponge_entry(half ? a.axh : a.ax, k - half * d.Px, d.nx, d.S, a.dx, a.dt, a.sv, a.sR, half);
+        return;
+    }
+    k -= 2 * d.Px;
+    if (k < 2 * d.Nz) {
+        const int half = k >= d.Nz;
+        sponge_entry(half ? a.azh : a.az, k - half * d.Nz, d.nz, d.S, a.dx, a.dt, a.sv, a.sR, half);
+        return;
+    }
+    k -= 2 * d.Nz;
+    if (k < a.ns) {
+        footprint_entry(a.src_xy, k, d, a.dx, a.src_scale, a.sidx, a.sw, a.status);
+        return;
+    }
+    k -= a.ns;
+    if (k < a.nr) footprint_entry(a.rec_xy, k, d, a.dx, 1.0, a.ridx, a.rw, a.status);
+}
+
 // Receiver footprints that share a cell, chained for a deterministic adjoint injection:
 // entry k (receiver k/4, corner k%4) gets the next entry with the same cell (n4 if none) in
-// bits 0..29, and bit 30 set when no earlier entry has its cell.  O(n4^2), run once.
+// bits 0..29, and bit 30 set when no earlier entry has its cell.  O(n4^2), run once; the cells go
+// through shared memory (from L2 one by one: 78 us for 256 receivers).
 constexpr int CHAIN_FIRST = 1 << 30;
+constexpr int CHAIN_NT = 128;
 
-__global__ void k_receiver_chain(const long long *__restrict__ idx, int n4, int *__restrict__ rl)
+__global__ void __launch_bounds__(CHAIN_NT) k_receiver_chain(const long long *__restrict__ idx, int n4, int *__restrict__ rl)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n4) return;
-    const long long c = idx[k];
+    __shared__ long long sc[8 * CHAIN_NT];
+    const int k = blockIdx.x * CHAIN_NT + threadIdx.x;
+    const long long c = k < n4 ? idx[k] : -1;
     bool first = true;
-    for (int m = 0; m < k && first; ++m) first = idx[m] != c;
     int nx = n4;
-    for (int m = k + 1; m < n4; ++m)
-        if (idx[m] == c) { nx = m; break; }
-    rl[k] = nx | (first ? CHAIN_FIRST : 0);
+    for (int m0 = 0; m0 < n4; m0 += 8 * CHAIN_NT) {
+        __syncthreads();
+        const int cnt = min(8 * CHAIN_NT, n4 - m0);
+        for (int m = threadIdx.x; m < cnt; m += CHAIN_NT) sc[m] = idx[m0 + m];
+        __syncthreads();
+        if (nx < n4 && !first) continue;
+        const int lo = min(cnt, max(0, k - m0)), hi = min(cnt, max(0, k + 1 - m0));   // entries before, up to k
+        for (int m = 0; m < lo && first; ++m) first = sc[m] != c;
+        for (int m = hi; m < cnt && nx == n4; ++m)
+            if (sc[m] == c) nx = m0 + m;
+    }
+    if (k < n4) rl[k] = nx | (first ? CHAIN_FIRST : 0);
 }
 
 // ------------------------------------------------------------ shared kernel arguments
@@ -392,46 +452,80 @@ __global__ void __launch_bounds__(FLUSH_X * FLUSH_Y) k_acc_flush(const float *__
     }
 }
 
-// Per padded cell, FP64, in place on the running sums of k_acc_flush:
-// gK = sum accK / K;  hx = g_bx * d bx/d rho_each = (sum accBx) bx^2/2 (g_bx = -sum accBx,
-// d bx / d rho = -bx^2/2 for each of its two cells), hz likewise.
-__global__ void k_grad_cells(const float *__restrict__ K, const float *__restrict__ bx,
-                             const float *__restrict__ bz, Dims d, double *__restrict__ gK,
-                             double *__restrict__ hx, double *__restrict__ hz)
+// The gradient's FP64 epilogue, in two passes over the running sums of k_acc_flush.  Per padded
+// cell, g_K = sK / K, and g_rho from the buoyancy nodes that touch it: h_x = g_bx * d bx/d rho_each
+// = sX bx^2/2 (g_bx = -sX, d bx / d rho = -bx^2/2 for each of its two cells), h_z likewise.  Every
+// physical cell takes the sum over the padded cells that copy it; corner cells copy into
+// (S + 1)^2 of them, which one thread each took 0.57 ms to walk, so the sums go one axis at a time.
+//
+// Pass 1: rows of the padded grid folded along x into fold[0..1][Nz][nx] (g_K, g_rho); one block
+// a row, a warp for each of the two edge columns.
+constexpr int FOLD_NT = 128;
+
+__global__ void __launch_bounds__(FOLD_NT) k_grad_fold(const float *__restrict__ K, const float *__restrict__ bx,
+                                                       const float *__restrict__ bz, Dims d, const double *__restrict__ sK,
+                                                       const double *__restrict__ sX, const double *__restrict__ sZ,
+                                                       double *__restrict__ fold)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= d.Nx || j >= d.Nz) return;
-    const long long m = cell(d, i, j);
-    const double b1 = bx[m], b2 = bz[m];
-    gK[m] = gK[m] / (double)K[m];
-    hx[m] = 0.5 * b1 * b1 * hx[m];
-    hz[m] = 0.5 * b2 * b2 * hz[m];
+    const int j = blockIdx.x;
+    const long long plane = (long long)d.Nz * d.nx;
+    auto half_b2 = [](const float *b, long long m) { const double v = b[m]; return 0.5 * v * v; };
+    auto cellg = [&](int i, double &gk, double &gr) {
+        const long long m = cell(d, i, j);
+        gk = sK[m] / (double)K[m];
+        const double hx = half_b2(bx, m) * sX[m], hz = half_b2(bz, m) * sZ[m];
+        gr = hx + hz;                                              // buoyancy nodes at i+1/2, j+1/2
+        if (i > 0) gr += half_b2(bx, m - 1) * sX[m - 1];           // node at i-1/2
+        if (i == d.Nx - 1) gr += hx;                               // last node reuses rho_i twice
+        if (j > 0) gr += half_b2(bz, m - d.Px) * sZ[m - d.Px];
+        if (j == d.Nz - 1) gr += hz;
+    };
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < 2) {   // physical columns 0 and nx - 1: the sponge cells beside them too
+        const int lo = warp == 0 ? 0 : d.nx - 1 + d.S, hi = warp == 0 ? d.S : d.Nx - 1;
+        double a = 0.0, b = 0.0;
+        for (int i = lo + lane; i <= hi; i += 32) {
+            double gk, gr;
+            cellg(i, gk, gr);
+            a += gk;
+            b += gr;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(0xffffffffu, a, o);
+            b += __shfl_down_sync(0xffffffffu, b, o);
+        }
+        if (lane == 0) {
+            const long long q = (long long)j * d.nx + (warp == 0 ? 0 : d.nx - 1);
+            fold[q] = a;
+            fold[plane + q] = b;
+        }
+        return;
+    }
+    for (int pi = 1 + (int)threadIdx.x - 64; pi < d.nx - 1; pi += FOLD_NT - 64) {
+        double gk, gr;
+        cellg(pi + d.S, gk, gr);
+        fold[(long long)j * d.nx + pi] = gk;
+        fold[plane + (long long)j * d.nx + pi] = gr;
+    }
 }
 
-// Per physical cell: fold the padding it feeds, form g_rho from the buoyancy nodes that
-// touch each padded cell, then the chain rule of every parameterization at the cell's
-// (K, rho) (closed-form Jacobians of the maps of Table 1), written as grads[5][2][nz][nx].
-__global__ void k_grad_final(const double *__restrict__ gK, const double *__restrict__ hx,
-                             const double *__restrict__ hz, const float *__restrict__ xa,
+// Pass 2: folds along z, then the chain rule of every parameterization at the cell's (K, rho)
+// (closed-form Jacobians of the maps of Table 1), written as grads[5][2][nz][nx].
+__global__ void k_grad_final(const double *__restrict__ fold, const float *__restrict__ xa,
                              const float *__restrict__ xb, int pz, double vp_o, double rho_o, Dims d,
                              double *__restrict__ grads)
 {
     const int pi = blockIdx.x * blockDim.x + threadIdx.x, pj = blockIdx.y * blockDim.y + threadIdx.y;
     if (pi >= d.nx || pj >= d.nz) return;
-    const int ilo = pi == 0 ? 0 : pi + d.S, ihi = pi == d.nx - 1 ? d.Nx - 1 : pi + d.S;
     const int jlo = pj == 0 ? 0 : pj + d.S, jhi = pj == d.nz - 1 ? d.Nz - 1 : pj + d.S;
+    const double *fK = fold + pi, *fR = fold + (long long)d.Nz * d.nx + pi;
     double sK = 0.0, sR = 0.0;
-    for (int j = jlo; j <= jhi; ++j)
-        for (int i = ilo; i <= ihi; ++i) {
-            const long long m = cell(d, i, j);
-            sK += gK[m];
-            double gr = hx[m] + hz[m];                       // buoyancy nodes at i+1/2, j+1/2
-            if (i > 0) gr += hx[m - 1];                      // node at i-1/2
-            if (i == d.Nx - 1) gr += hx[m];                  // last node reuses rho_i twice
-            if (j > 0) gr += hz[m - d.Px];
-            if (j == d.Nz - 1) gr += hz[m];
-            sR += gr;
-        }
+#pragma unroll 8
+    for (int j = jlo; j <= jhi; ++j) {
+        sK += fK[(long long)j * d.nx];
+        sR += fR[(long long)j * d.nx];
+    }
     const long long q = (long long)pj * d.nx + pi;
     double K, rho;
     kr_of(pz, xa[q], xb[q], vp_o, rho_o, K, rho);
