@@ -956,6 +956,11 @@ int fwi_born(const fwi_grid *g, fwi_param pz, const float *xi_a, const float *xi
     for (int gi = 0; gi < P.ngroups; ++gi) {
         TraceRange tr(PH_BORN);
         const int s0 = gi * P.B, bg = std::min(P.B, P.ns - s0);
+        ResPlan rp;
+        if (res_wanted(P, RES_BORN, bg, rp)) {
+            if ((rc = res_born(P, work, st, src->wavelet, rp, s0, bg, dtraces + (size_t)s0 * P.nr * P.nt))) return rc;
+            continue;
+        }
         const size_t bf = (size_t)bg * d.Np * sizeof(float);
         for (size_t off : {P.p[0], P.vx[0], P.vz[0], P.dp[0], P.dvx[0], P.dvz[0]})
             CK(cudaMemsetAsync(at<char>(work, off), 0, bf, st));

@@ -102,7 +102,8 @@ __device__ __forceinline__ float4 row_diff(const float4 &a, const float4 &b, con
 
 struct ResFwdArgs {
     const float *p0, *vx0, *vz0;    // state before step n0 of shot 0 (null: zero)
-    float *p1, *vx1, *vz1;          // state after step n1 - 1 (null: not written)
+    float *p1, *vx1, *vz1;          // state after step n1 - 1 (null: not written); may be the
+                                    // state before (every step exchanges: a neighbour has read it)
     float *hist;                    // p^{n0} .. p^{n1}, one slot a step (null: not kept)
     long long slot;                 // floats between history slots
     Model mo;
@@ -128,6 +129,28 @@ __device__ __forceinline__ void mail_put4(unsigned long long *m, const float4 &v
     asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(m + 2), "l"(t | __float_as_uint(v.z)),
                  "l"(t | __float_as_uint(v.w))
                  : "memory");
+}
+
+// The jobs of a launch: job j takes blocks start[j] .. start[j + 1) (tiles within shots).  A single
+// call's launch has CAP 1.
+constexpr int RES_CAP = 24;
+template <class A, int CAP>
+struct ResBatch {
+    int njobs;
+    int start[CAP + 1];
+    A jobs[CAP];
+};
+
+template <class A, int CAP>
+__device__ __forceinline__ const A &res_job(const ResBatch<A, CAP> &t, int &block)
+{
+    int j = 0;
+    block = blockIdx.x;
+    if constexpr (CAP > 1) {
+        while (j + 1 < t.njobs && t.start[j + 1] <= block) ++j;
+        block -= t.start[j];
+    }
+    return t.jobs[j];
 }
 
 struct MailWord4 {
@@ -353,28 +376,32 @@ __device__ __forceinline__ void warp_sides(const float4 &b, float4 &l, float4 &r
     if (M > 3) r.z = __shfl_down_sync(all, b.z, 1);
 }
 
-// component i of v += kw * w, product and sum rounded apart (as the streaming kernels' injection)
+// Component i of v += kw * w: with product and sum rounded apart, or together (FUSED).  Which, is what
+// the compiler made of the streaming kernels' injection, whose results these kernels reproduce.
+template <bool FUSED>
 __device__ __forceinline__ void add_source(float4 &v, int i, float kw, float w)
 {
-    const float a = __fmul_rn(kw, w);
-    v.x = i == 0 ? __fadd_rn(v.x, a) : v.x;
-    v.y = i == 1 ? __fadd_rn(v.y, a) : v.y;
-    v.z = i == 2 ? __fadd_rn(v.z, a) : v.z;
-    v.w = i == 3 ? __fadd_rn(v.w, a) : v.w;
+    auto add = [&](float x) { return FUSED ? fmaf(kw, w, x) : __fadd_rn(x, __fmul_rn(kw, w)); };
+    v.x = i == 0 ? add(v.x) : v.x;
+    v.y = i == 1 ? add(v.y) : v.y;
+    v.z = i == 2 ? add(v.z) : v.z;
+    v.w = i == 3 ? add(v.w) : v.w;
 }
 
 // Forward steps n0 .. n1 - 1.
-template <class S>
-__global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant__ ResFwdArgs a)
+template <class S, int CAP>
+__global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant__ ResBatch<ResFwdArgs, CAP> t)
 {
     constexpr int M = S::M, R = S::R, HR = S::HR, PP = S::PP, PZ = S::PZ;
     extern __shared__ __align__(16) unsigned char fwi_smem[];
     ResFwdSmem<S> &sh = *reinterpret_cast<ResFwdSmem<S> *>(fwi_smem);
+    int block;
+    const ResFwdArgs &a = res_job(t, block);
     const ResCut &c = a.cut;
     const Dims &d = a.d;
     const Model &mo = a.mo;
     const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
-    const ResTile T = res_tile(c, blockIdx.x);
+    const ResTile T = res_tile(c, block);
     const long long so = (long long)T.s * d.Np;
     int *stt = mo.status;
 
@@ -496,7 +523,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
                     for (int k = 0; k < 4; ++k) {
                         const int e = e0 + r, i = sh.si[k] - 4 * g;
                         if (sh.sj[k] == e && e >= 0 && e < T.h && i >= 0 && i < 4)
-                            add_source(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
+                            add_source<false>(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
                     }
             send.put(T, slot, e0, p, tag);
             if (own) {
@@ -549,12 +576,12 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
             for (int r = 0; r < R; ++r)
                 if (!own || e0 + r < 0 || e0 + r >= T.h) p[r] = ld4(prow + r * PP);
     }
-    if (a.p1)
+    if (a.vx1)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int e = e0 + r, o = go + r * d.Px;
             if (FWI_IN(own && e >= 0 && e < T.h, o, 4, d.Np, stt)) {
-                st4(a.p1 + so + o, p[r]);
+                if (a.p1) st4(a.p1 + so + o, p[r]);
                 st4(a.vx1 + so + o, vx[r]);
                 st4(a.vz1 + so + o, vz[r]);
             }
@@ -576,7 +603,8 @@ using ResAdj4 = ResShape<4, 4, 12>;
 
 struct ResAdjArgs {
     const float *ap0, *avx0, *avz0;   // pbar^{nhi+1} (injected), vbar of the launch's shots
-    float *ap1, *avx1, *avz1;         // pbar^{nlo}, vbar after step nlo (other buffers)
+    float *ap1, *avx1, *avz1;         // pbar^{nlo}, vbar after step nlo; other buffers, or with two
+                                      // steps or more (one exchange) the same
     const float *pn;                  // p^{nlo}, one slot a step
     long long slot;
     float *accK, *accBx, *accBz;      // FP32 accumulators, read and written once
@@ -618,17 +646,19 @@ __device__ __forceinline__ float4 add_ftz(const float4 &a, const float4 &v)
     return r;
 }
 
-template <class S>
-__global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant__ ResAdjArgs a)
+template <class S, int CAP>
+__global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant__ ResBatch<ResAdjArgs, CAP> t)
 {
     constexpr int M = S::M, R = S::R, HR = S::HR, PP = S::PP, PZ = S::PZ;
     extern __shared__ __align__(16) unsigned char fwi_smem[];
     ResAdjSmem<S> &sh = *reinterpret_cast<ResAdjSmem<S> *>(fwi_smem);
+    int block;
+    const ResAdjArgs &a = res_job(t, block);
     const ResCut &c = a.cut;
     const Dims &d = a.d;
     const Model &mo = a.mo;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
-    const ResTile T = res_tile(c, blockIdx.x);
+    const ResTile T = res_tile(c, block);
     const long long so = (long long)T.s * d.Np;
     int *stt = mo.status;
 
@@ -862,6 +892,297 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
             st4(a.accBz + so + o, ld4(accz + r * 128));
         }
     }
+}
+
+// ------------------------------------------------------------------------ Born steps (S6)
+//
+// Background and scattered wavefields (see k_born_warp) stepped together on chip: the forward
+// kernel's structure with two of everything.  Three rows a warp; the model's perturbation sits in
+// shared memory, read by its own lane alone.
+using ResBorn2 = ResShape<2, 3, 12>;
+using ResBorn4 = ResShape<4, 3, 12>;
+
+struct ResBornArgs {
+    const float *p0, *vx0, *vz0, *q0, *ux0, *uz0;   // state before step n0 of shot 0 (null p0: zero)
+    float *p1, *vx1, *vz1, *q1, *ux1, *uz1;         // state after step n1 - 1 (null p1: not written); may
+                                                    // be the state before
+    Model mo;
+    Pert pe;
+    Dims d;
+    ResStencil st;
+    Source src;
+    const long long *ridx;
+    const float *rw;
+    float *traces;                                  // [shots][nr][nt], samples of q (null: none)
+    int nr, nt;
+    int n0, n1;
+    ResCut cut;
+    unsigned long long *mail, *mailq;               // p's and q's mailboxes
+};
+
+template <class S>
+struct __align__(16) ResBornSmem {
+    float p[S::E + S::HR][S::PP], q[S::E + S::HR][S::PP];            // row e at [e + HR]
+    float vz[S::E + 2 * S::M][S::PZ], uz[S::E + 2 * S::M][S::PZ];    // row e at [e + 2M]
+    float dm[3][S::E][128];                  // dK, dbx, dbz: row e at [e + M], lane l at 4 l
+    float2 az[S::E], azh[S::E];
+    int sj[4], si[4];
+    float sw[4];
+    ResRec rec;
+    int abort;
+};
+
+template <class S, int CAP>
+__global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constant__ ResBatch<ResBornArgs, CAP> t)
+{
+    constexpr int M = S::M, R = S::R, HR = S::HR, PP = S::PP, PZ = S::PZ;
+    extern __shared__ __align__(16) unsigned char fwi_smem[];
+    ResBornSmem<S> &sh = *reinterpret_cast<ResBornSmem<S> *>(fwi_smem);
+    int block;
+    const ResBornArgs &a = res_job(t, block);
+    const ResCut &c = a.cut;
+    const Dims &d = a.d;
+    const Model &mo = a.mo;
+    const int tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
+    const ResTile T = res_tile(c, block);
+    const long long so = (long long)T.s * d.Np;
+    int *stt = mo.status;
+
+    for (int k = tid; k < (int)(sizeof(ResBornSmem<S>) / 4); k += nt) reinterpret_cast<int *>(fwi_smem)[k] = 0;
+    __syncthreads();
+    for (int k = tid; k < S::E; k += nt) {
+        const int j = T.z0 - M + k;
+        if (j >= 0 && j < d.Nz) {
+            sh.az[k] = make_float2(mo.az[j], mo.az[j]);
+            sh.azh[k] = make_float2(mo.azh[j], mo.azh[j]);
+        }
+    }
+    if (tid < 4) {
+        const long long o = a.src.idx[4 * T.s + tid];
+        sh.sj[tid] = (int)(o / d.Px) - T.z0;
+        sh.si[tid] = (int)(o % d.Px) - 4 * T.g0;
+        sh.sw[tid] = a.src.w[4 * T.s + tid];
+    }
+    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid);
+    float *const p00 = &sh.p[HR][8], *const q00 = &sh.q[HR][8];
+    if (a.p0)   // initial fields of the tile and its halo
+        for (int k = tid; k < (T.h + 2 * HR) * (T.ng + 4); k += nt) {
+            const int row = k / (T.ng + 4) - HR, g = k % (T.ng + 4) - 2;
+            const int j = T.z0 + row, i = 4 * (T.g0 + g);
+            const bool rin = row >= 0 && row < T.h, gin = g >= 0 && g < T.ng;
+            if (!rin && !gin) continue;
+            if (FWI_IN(j >= 0 && j < d.Nz && i >= 0 && i < d.Nx, j * d.Px + i, 4, d.Np, stt)) {
+                st4(p00 + row * PP + 4 * g, ld4(a.p0 + so + j * d.Px + i));
+                st4(q00 + row * PP + 4 * g, ld4(a.q0 + so + j * d.Px + i));
+            }
+        }
+    __syncthreads();
+
+    const int g = lane - 1, e0 = (tid >> 5) * R - M, col = 4 * (T.g0 + g);
+    const bool own = g >= 0 && g < T.ng, side = (g == -1 || g == T.ng) && col >= 0 && col < d.Nx;
+    const int go = (T.z0 + e0) * d.Px + col;
+    const float4 axv = ldg_if(mo.ax + col, own), axhv = ldg_if(mo.axh + col, own || side);
+    float4 p[R], vx[R], vz[R], q[R], ux[R], uz[R], Kv[R], bx[R], bz[R];
+    float *const dk = &sh.dm[0][e0 + M][4 * lane], *const dbx = &sh.dm[1][e0 + M][4 * lane], *const dbz = &sh.dm[2][e0 + M][4 * lane];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = e0 + r, j = T.z0 + e, o = go + r * d.Px;
+        const bool grid = j >= 0 && j < d.Nz, rin = e >= 0 && e < T.h, zin = e < T.h + M - 1;
+        const bool fx = FWI_IN(grid && rin && (own || side), o, 4, d.Np, stt), fz = FWI_IN(grid && zin && own, o, 4, d.Np, stt);
+        Kv[r] = ldg_if(mo.K + o, fz && rin);
+        bx[r] = ldg_if(mo.bx + o, fx);
+        bz[r] = ldg_if(mo.bz + o, fz);
+        st4(dk + r * 128, ldg_if(a.pe.dK + o, fz && rin));
+        st4(dbx + r * 128, ldg_if(a.pe.dbx + o, fx));
+        st4(dbz + r * 128, ldg_if(a.pe.dbz + o, fz));
+        p[r] = vx[r] = vz[r] = q[r] = ux[r] = uz[r] = f4(0.f);
+        if (a.p0) {
+            if (fx) {
+                vx[r] = ld4(a.vx0 + so + o);
+                ux[r] = ld4(a.ux0 + so + o);
+            }
+            if (fz) {
+                vz[r] = ld4(a.vz0 + so + o);
+                uz[r] = ld4(a.uz0 + so + o);
+            }
+            p[r] = ld4(p00 + e * PP + 4 * g);
+            q[r] = ld4(q00 + e * PP + 4 * g);
+        }
+    }
+    bool hsrc = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        hsrc |= own && sh.si[k] >= 4 * g && sh.si[k] < 4 * g + 4 && sh.sj[k] >= max(e0, 0) && sh.sj[k] < min(e0 + R, T.h);
+    const long long tile = (long long)T.s * c.tx * c.tz + T.t;
+    unsigned long long *const boxp = a.mail + tile * S::MAIL, *const boxq = a.mailq + tile * S::MAIL;
+    const ResSend<S> sendp(boxp, T, c, g, e0), sendq(boxq, T, c, g, e0);
+    const ResRecv<S> recv(T, tid, nt);
+    float *const prow = p00 + e0 * PP + 4 * g, *const qrow = q00 + e0 * PP + 4 * g;
+    float *const vrow = &sh.vz[e0 + 2 * M][4 * lane], *const urow = &sh.uz[e0 + 2 * M][4 * lane];
+    const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
+    const float2 *const nc = a.st.nc;
+    const bool inner = e0 >= 0 && e0 + R <= T.h;
+
+    float wn = hsrc ? __ldg(a.src.wav + a.n0) : 0.f;
+    for (int n = a.n0; n < a.n1; ++n) {
+        // ---------------------------------------------------------------- velocities
+        {
+            float4 gp[R];
+            {
+                float4 w[R + HR];
+#pragma unroll
+                for (int k = 0; k < M - 1; ++k) w[k] = ld4(prow + (k - (M - 1)) * PP);
+#pragma unroll
+                for (int k = 0; k < R; ++k) w[M - 1 + k] = p[k];
+#pragma unroll
+                for (int k = 0; k < M; ++k) w[M - 1 + R + k] = ld4(prow + (R + k) * PP);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    gp[r] = f4(0.f);
+#pragma unroll
+                    for (int k = 1; k <= M; ++k) gp[r] = rtap(nc[k - 1], w[r + M - 1 + k], w[r + M - k], gp[r]);
+                }
+            }
+            float4 w[R + HR];
+#pragma unroll
+            for (int k = 0; k < M - 1; ++k) w[k] = ld4(qrow + (k - (M - 1)) * PP);
+#pragma unroll
+            for (int k = 0; k < R; ++k) w[M - 1 + k] = q[k];
+#pragma unroll
+            for (int k = 0; k < M; ++k) w[M - 1 + R + k] = ld4(qrow + (R + k) * PP);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 gq = f4(0.f);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) gq = rtap(nc[k - 1], w[r + M - 1 + k], w[r + M - k], gq);
+                const float4 fz = rscale(azhr[r], axv);
+                vz[r] = pmul(fz, pfma(bz[r], gp[r], vz[r]));
+                uz[r] = pmul(fz, pfma(ld4(dbz + r * 128), gp[r], pfma(bz[r], gq, uz[r])));
+                st4(vrow + r * PZ, vz[r]);
+                st4(urow + r * PZ, uz[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 gpx = row_diff<M, true>(ld4(prow + r * PP - 4), p[r], ld4(prow + r * PP + 4), nc);
+            const float4 gqx = row_diff<M, true>(ld4(qrow + r * PP - 4), q[r], ld4(qrow + r * PP + 4), nc);
+            const float4 fx = rscale(azr[r], axhv);
+            vx[r] = pmul(fx, pfma(bx[r], gpx, vx[r]));
+            ux[r] = pmul(fx, pfma(ld4(dbx + r * 128), gpx, pfma(bx[r], gqx, ux[r])));
+        }
+        __syncthreads();
+        // ------------------------------------------------------------------ pressure
+        const unsigned tag = (unsigned)(n - a.n0) + 1u;
+        const int slot = (n & 1) * S::SLOT;
+        {
+            float4 dv[R];
+            {
+                float4 w[R + HR];
+#pragma unroll
+                for (int k = 0; k < M; ++k) w[k] = ld4(vrow + (k - M) * PZ);
+#pragma unroll
+                for (int k = 0; k < R; ++k) w[M + k] = vz[k];
+#pragma unroll
+                for (int k = 0; k < M - 1; ++k) w[M + R + k] = ld4(vrow + (R + k) * PZ);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    float4 l, rr;
+                    warp_sides<M>(vx[r], l, rr);
+                    dv[r] = row_diff<M, false>(l, vx[r], rr, nc);
+#pragma unroll
+                    for (int k = 1; k <= M; ++k) dv[r] = rtap(nc[k - 1], w[r + M + k - 1], w[r + M - k], dv[r]);
+                }
+            }
+            float4 w[R + HR];
+#pragma unroll
+            for (int k = 0; k < M; ++k) w[k] = ld4(urow + (k - M) * PZ);
+#pragma unroll
+            for (int k = 0; k < R; ++k) w[M + k] = uz[k];
+#pragma unroll
+            for (int k = 0; k < M - 1; ++k) w[M + R + k] = ld4(urow + (R + k) * PZ);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                float4 l, rr;
+                warp_sides<M>(ux[r], l, rr);
+                float4 du = row_diff<M, false>(l, ux[r], rr, nc);
+#pragma unroll
+                for (int k = 1; k <= M; ++k) du = rtap(nc[k - 1], w[r + M + k - 1], w[r + M - k], du);
+                const float4 fp = rscale(azr[r], axv);
+                p[r] = pmul(fp, pfma(Kv[r], dv[r], p[r]));
+                q[r] = pmul(fp, pfma(ld4(dk + r * 128), dv[r], pfma(Kv[r], du, q[r])));
+            }
+        }
+        if (hsrc) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int e = e0 + r, i = sh.si[k] - 4 * g;
+                    if (sh.sj[k] == e && e >= 0 && e < T.h && i >= 0 && i < 4) {
+                        add_source<true>(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
+                        add_source<true>(q[r], i, __fmul_rn((dk + r * 128)[i], wn), sh.sw[k]);
+                    }
+                }
+            if (n + 1 < a.n1) wn = __ldg(a.src.wav + n + 1);
+        }
+        sendp.put(T, slot, e0, p, tag);
+        sendq.put(T, slot, e0, q, tag);
+        if (own)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (inner || (e0 + r >= 0 && e0 + r < T.h)) {
+                    st4(prow + r * PP, p[r]);
+                    st4(qrow + r * PP, q[r]);
+                }
+        // ------------------------------------------------------------------ exchange
+        if (e0 <= 0 && e0 + R > 0 && g == 0 && T.U && T.L) {   // the first cell of q, for the diagonal tile's samples
+            float v = 0.f;
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (e0 + r == 0) v = q[r].x;
+            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(boxq - (long long)(c.tx + 1) * S::MAIL + 2 * S::SLOT + (n & 3)),
+                         "l"((unsigned long long)tag << 32 | __float_as_uint(v))
+                         : "memory");
+        }
+        bool ok = recv.get(boxp + slot, T, p00, tag, tid, nt);
+        ok = recv.get(boxq + slot, T, q00, tag, tid, nt) && ok;
+        if (tid == 0 && sh.rec.diag && T.R && T.D) {
+            unsigned long long v = 0;
+            int spin = 0;
+            do {
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(boxq + 2 * S::SLOT + (n & 3)) : "memory");
+            } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
+            ok = ok && spin < RES_SPIN;
+            q00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
+        }
+        if (!ok) {
+            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
+            atomicOr(stt, ST_ETIMEOUT);
+        }
+        __syncthreads();
+        if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
+        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, q00, PP, tid);
+        if (!own || !inner)
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if (!own || e0 + r < 0 || e0 + r >= T.h) {
+                    p[r] = ld4(prow + r * PP);
+                    q[r] = ld4(qrow + r * PP);
+                }
+    }
+    if (a.p1)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int e = e0 + r, o = go + r * d.Px;
+            if (FWI_IN(own && e >= 0 && e < T.h, o, 4, d.Np, stt)) {
+                st4(a.p1 + so + o, p[r]);
+                st4(a.vx1 + so + o, vx[r]);
+                st4(a.vz1 + so + o, vz[r]);
+                st4(a.q1 + so + o, q[r]);
+                st4(a.ux1 + so + o, ux[r]);
+                st4(a.uz1 + so + o, uz[r]);
+            }
+        }
 }
 
 }  // namespace fwi

@@ -119,6 +119,55 @@ def test_adjoint_is_bitwise_the_streaming_kernels(F, nx, nz, order, sponge):
     assert torch.equal(ref, got)
 
 
+@pytest.mark.parametrize("nx,nz,order,sponge", GRIDS)
+def test_born_is_bitwise_the_streaming_kernels(F, nx, nz, order, sponge):
+    w = case(nx, nz, order, sponge)
+    hi = np.array([(nx - 1) * w.dx, (nz - 1) * w.dx])
+    w.rec_xy = np.concatenate([w.rec_xy, (hi * np.random.default_rng(3).random((90, 2))).astype(np.float32)])
+    g = gpu_grid(w)
+    da, db = (I.random_like(w.xi_a.shape, s, 0.05) for s in (1, 2))
+    ref, got = both(F, lambda: F.fwi_born(g, w.pz, w.xi_a, w.xi_b, da, db, w.src_xy, w.wavelet, w.rec_xy), "k_res_born")
+    assert ref.abs().max().item() > 0
+    assert torch.equal(ref, got)
+
+
+@pytest.mark.parametrize("iterations", [1, 9, 64, 256])
+def test_engine_runs_on_chip_equal_single_calls(F, iterations):
+    """Runs of steps between engine calls of any length (odd remainders stream), several shot groups,
+    checkpointed gradients with recomputation, jobs spread over launches."""
+    from paper_1804_01184_gb300 import engine
+    E = engine.Engine(2 << 30)
+    E.arena.fill_(0xFF)
+    want = []
+    for k in range(9):
+        w = I.small_case(seed=900 + k, nx=60 + 23 * k, nz=150 - 11 * k, nt=90 + 7 * k, order=4 if k % 4 == 3 else 8, sponge=6,
+                         ns=2 + k % 4, nr=8)
+        g = gpu_grid(w)
+        ar = (g, w.pz, w.xi_a, w.xi_b)
+        tail = (w.src_xy, w.wavelet, w.rec_xy)
+        budget = 0 if k % 2 else 1 << 28
+        op = (F.OP_MODEL, F.OP_BORN, F.OP_GRADIENT)[k % 3]
+        work = torch.empty(F.fwi_workspace_bytes(g, w.ns, w.nr, op, budget), dtype=torch.uint8, device="cuda")
+        if op == F.OP_MODEL:
+            want.append((E.submit_model(*ar, *tail, work_budget=budget), F.fwi_model(*ar, *tail, work=work)))
+        elif op == F.OP_BORN:
+            d = tuple(I.random_like(w.xi_a.shape, 40 + k + s, 0.05) for s in (0, 1))
+            want.append((E.submit_born(*ar, *d, *tail, work_budget=budget), F.fwi_born(*ar, *d, *tail, work=work)))
+        else:
+            data = I.random_like((w.ns, w.nr, w.nt), 50 + k, 1.0)
+            want.append((E.submit_gradient(*ar, *tail, data, work_budget=budget),
+                         F.fwi_gradient(*ar, *tail, data, work=work)))
+    (res, used) = kernels(F, lambda: {r.ticket: r for r in E.drain(iterations)})
+    if iterations >= 64:
+        assert any("k_res" in k for k in used), used
+    for t, ref in want:
+        r = res[t]
+        got = (r.traces,) if r.traces is not None else (r.misfit, r.grads)
+        for x, y in zip(got, ref if isinstance(ref, tuple) else (ref,)):
+            assert torch.equal(x, y)
+    E.close()
+
+
 def test_more_shots_than_a_launch_holds(F):
     w = case(201, 201, 8, 40, ns=33, nr=20, nt=30)
     g = gpu_grid(w)
