@@ -1064,7 +1064,42 @@ int fwi_misfit_weighted(const float *traces, const float *data, long long ntrace
     if (ntraces < 0 || nt < 1 || !misfit || (ntraces > 0 && (!traces || !data)))
         return fail(FWI_EINVAL, "invalid misfit arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LAUNCH(fwi::k_misfit, 1, fwi::RED_THREADS, 0, st, traces, data, ntraces * nt, weights, nt, misfit);
+    // one cluster: 16 blocks where the device runs such clusters, 8 (portable) elsewhere
+    static const int wide = [] {
+        cudaLaunchConfig_t c = {};
+        cudaLaunchAttribute at[1];
+        c.gridDim = dim3(16);
+        c.blockDim = dim3(fwi::MISFIT_NT);
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {16, 1, 1};
+        c.attrs = at;
+        c.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(fwi::k_misfit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, fwi::k_misfit, &c) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        return n > 0 ? 16 : 8;
+    }();
+    const long long n = ntraces * nt;
+    // small sums: no more blocks than there are four elements a thread for
+    unsigned nb = 1;
+    while (nb < (unsigned)wide && n > 4LL * fwi::MISFIT_NT * nb) nb *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {nb, 1, 1};
+    cfg.gridDim = dim3(nb);
+    cfg.blockDim = dim3(fwi::MISFIT_NT);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaEvent_t *ev = g_prof.next("fwi::k_misfit");
+    if (ev) cudaEventRecord(ev[0], st);
+    CK(cudaLaunchKernelEx(&cfg, fwi::k_misfit, traces, data, n, weights, nt, misfit));
+    if (ev) cudaEventRecord(ev[1], st);
+    ++g_launches;
     return finish(st);
 }
 

@@ -41,11 +41,6 @@ struct ResShape {
     static constexpr int E = NW * R, H = E - HR;     // extended rows (from -M on), own rows
     static constexpr int PP = W + 16;                // pitch of a p row: column c at c + 8
     static constexpr int PZ = 128;                   // pitch of a v_z row: lane l at 4 l
-    // mailbox slot, in words: 2M - 1 rows from above and below, 8 columns from the left and right
-    static constexpr int MB = HR * W, ML = 2 * HR * W, MR = ML + 8 * H, SLOT = MR + 8 * H;
-    // two slots and a ring of 4 for the lower right diagonal tile's first cell (diagonal tiles
-    // do not wait on each other)
-    static constexpr int MAIL = 2 * SLOT + 4;
 };
 
 // Four rows a warp (five at 4th order, whose windows are shorter): 96 registers of fields and model a thread and room for the stencil windows
@@ -57,6 +52,33 @@ using ResFwd4 = ResShape<4, 4, 12>;
 // more than gbase (hbase).
 struct ResCut {
     int tx, tz, gbase, grem, hbase, hrem;
+};
+
+// A tile's mailbox, in words: two slots of 2M - 1 rows from above and below and 8 columns from the
+// left and right, and a ring of 4 for the lower right diagonal tile's first cell (diagonal
+// tiles do not wait on each other).  The engine's are sized for the cut's largest tile (half
+// a job's fields hold state while it runs); a single call's for the shape's, whose constants
+// save 2 to 5 % of a step.
+template <class S, bool FIT>
+struct ResMail {
+    int w, below, left, right, slot, all;    // pitch of a row; offsets in a slot; words of a slot, of a tile
+    __host__ __device__ explicit ResMail(const ResCut &c)
+    {
+        w = 4 * (c.gbase + (c.grem > 0));
+        const int h = c.hbase + (c.hrem > 0);
+        below = S::HR * w;
+        left = 2 * below;
+        right = left + 8 * h;
+        slot = right + 8 * h;
+        all = 2 * slot + 4;
+    }
+};
+
+template <class S>
+struct ResMail<S, false> {
+    static constexpr int w = S::W, below = S::HR * w, left = 2 * below, right = left + 8 * S::H, slot = right + 8 * S::H,
+                         all = 2 * slot + 4;
+    __host__ __device__ explicit ResMail(const ResCut &) {}
 };
 
 // The stencil's weights (negated: -c_k dt / dx) in both halves of a pair, as the packed
@@ -116,7 +138,7 @@ struct ResFwdArgs {
     int nr, nt;
     int n0, n1;
     ResCut cut;
-    unsigned long long *mail;       // [shots][tiles][MAIL] mailboxes, cleared before the launch
+    unsigned long long *mail;       // [shots][tiles] mailboxes (ResMail), cleared before the launch
 };
 
 // Four values and their step tag as two 16-byte stores; each 8-byte word is written whole.
@@ -131,8 +153,8 @@ __device__ __forceinline__ void mail_put4(unsigned long long *m, const float4 &v
                  : "memory");
 }
 
-// The jobs of a launch: job j takes blocks start[j] .. start[j + 1) (tiles within shots).  A single
-// call's launch has CAP 1.
+// What a launch works on: a single call's arguments (CAP 1), or the engine's table, whose job j
+// takes blocks start[j] .. start[j + 1) (tiles within shots).
 constexpr int RES_CAP = 24;
 template <class A, int CAP>
 struct ResBatch {
@@ -141,15 +163,25 @@ struct ResBatch {
     A jobs[CAP];
 };
 
+template <class A>
+struct ResBatch<A, 1> {
+    A job;
+};
+
+template <class A>
+__device__ __forceinline__ const A &res_job(const ResBatch<A, 1> &t, int &block)
+{
+    block = blockIdx.x;
+    return t.job;
+}
+
 template <class A, int CAP>
 __device__ __forceinline__ const A &res_job(const ResBatch<A, CAP> &t, int &block)
 {
     int j = 0;
     block = blockIdx.x;
-    if constexpr (CAP > 1) {
-        while (j + 1 < t.njobs && t.start[j + 1] <= block) ++j;
-        block -= t.start[j];
-    }
+    while (j + 1 < t.njobs && t.start[j + 1] <= block) ++j;
+    block -= t.start[j];
     return t.jobs[j];
 }
 
@@ -271,36 +303,36 @@ __device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, c
 
 // What a thread receives: the float4 tid, tid + nt, ... of the halo; the first two kept as
 // (mailbox word, offset from the field's own cell (0, 0)).
-template <class S>
+template <class S, class Mail>
 struct ResRecv {
     int n, w0, o0, w1, o1;
-    __device__ ResRecv(const ResTile &T, int tid, int nt)
+    __device__ ResRecv(const ResTile &T, const Mail &B, int tid, int nt)
     {
         n = (T.U + T.D) * S::HR * T.ng + 2 * (T.L + T.R) * T.h;
-        item(T, tid, w0, o0);
-        item(T, tid + nt, w1, o1);
+        item(T, B, tid, w0, o0);
+        item(T, B, tid + nt, w1, o1);
     }
-    __device__ __forceinline__ void item(const ResTile &T, int k, int &word, int &off) const
+    __device__ __forceinline__ void item(const ResTile &T, const Mail &B, int k, int &word, int &off) const
     {
         const int nrow = S::HR * T.ng, nU = T.U ? nrow : 0, nD = T.D ? nrow : 0, nL = T.L ? 2 * T.h : 0;
         if (k >= n) k = 0;
         if (k < nU + nD) {
             const bool up = k < nU;
             const int q = up ? k : k - nU, r = q / T.ng, g = 4 * (q - r * T.ng);
-            word = (up ? 0 : S::MB) + r * S::W + g;
+            word = (up ? 0 : B.below) + r * B.w + g;
             off = ((up ? -S::HR : T.h) + r) * S::PP + g;
         } else {
             k -= nU + nD;
             const bool left = k < nL;
             if (!left) k -= nL;
-            word = (left ? S::ML : S::MR) + 4 * k;
+            word = (left ? B.left : B.right) + 4 * k;
             off = (k >> 1) * S::PP + (left ? -8 : 4 * T.ng) + 4 * (k & 1);
         }
     }
     // words of step `tag` of this tile's mailbox slot m into the halo of the field whose own cell
     // (0, 0) is at p; false when a wait expired
-    __device__ __forceinline__ bool get(const unsigned long long *m, const ResTile &T, float *p, unsigned tag, int tid,
-                                        int nt) const
+    __device__ __forceinline__ bool get(const unsigned long long *m, const ResTile &T, const Mail &B, float *p,
+                                        unsigned tag, int tid, int nt) const
     {
         int spin = 0;
         if (tid < n) {
@@ -316,7 +348,7 @@ struct ResRecv {
             }
             for (int k = tid + 2 * nt; k < n; k += nt) {
                 int w, o;
-                item(T, k, w, o);
+                item(T, B, k, w, o);
                 mail_get4(m + w, a);
                 while (!mail_ready(a, tag) && ++spin < RES_SPIN) mail_get4(m + w, a);
                 st4(p + o, mail_value(a));
@@ -328,22 +360,22 @@ struct ResRecv {
 
 // What a lane sends of its own rows: up and down (rows within HR of the edge), and left or right
 // (the two groups at the edge; tiles with such a neighbour have at least 4 groups).
-template <class S>
+template <class S, class Mail>
 struct ResSend {
     unsigned long long *ud, *lr;         // word of row 0 in the neighbour's slot; null: none
     int dn;                              // down's offset from up
     bool up, down;                       // this warp has rows for the neighbour
-    __device__ ResSend(unsigned long long *box, const ResTile &T, const ResCut &c, int g, int e0)
+    __device__ ResSend(unsigned long long *box, const ResTile &T, const ResCut &c, const Mail &B, int g, int e0)
     {
         const bool own = g >= 0 && g < T.ng;
         up = own && T.U && e0 < S::HR && e0 + S::R > 0;
         down = own && T.D && e0 + S::R > T.h - S::HR && e0 < T.h;
-        ud = box - (long long)c.tx * S::MAIL + S::MB + 4 * g;
-        dn = 2 * c.tx * S::MAIL - S::MB - (T.h - S::HR) * S::W;
-        lr = own && T.L && g < 2 ? box - S::MAIL + S::MR + 4 * g
-             : own && T.R && g >= T.ng - 2 ? box + S::MAIL + S::ML + 4 * (g - (T.ng - 2)) : nullptr;
+        ud = box - (long long)c.tx * B.all + B.below + 4 * g;
+        dn = 2 * c.tx * B.all - B.below - (T.h - S::HR) * B.w;
+        lr = own && T.L && g < 2 ? box - B.all + B.right + 4 * g
+             : own && T.R && g >= T.ng - 2 ? box + B.all + B.left + 4 * (g - (T.ng - 2)) : nullptr;
     }
-    __device__ __forceinline__ void put(const ResTile &T, int slot, int e0, const float4 (&v)[S::R], unsigned tag) const
+    __device__ __forceinline__ void put(const ResTile &T, const Mail &B, int slot, int e0, const float4 (&v)[S::R], unsigned tag) const
     {
         constexpr int R = S::R;
         if (lr)
@@ -353,11 +385,11 @@ struct ResSend {
         if (up)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (e0 + r >= 0 && e0 + r < S::HR) mail_put4(ud + slot + (e0 + r) * S::W, v[r], tag);
+                if (e0 + r >= 0 && e0 + r < S::HR) mail_put4(ud + slot + (e0 + r) * B.w, v[r], tag);
         if (down)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (e0 + r >= T.h - S::HR && e0 + r < T.h) mail_put4(ud + dn + slot + (e0 + r) * S::W, v[r], tag);
+                if (e0 + r >= T.h - S::HR && e0 + r < T.h) mail_put4(ud + dn + slot + (e0 + r) * B.w, v[r], tag);
     }
 };
 
@@ -459,9 +491,11 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         hsrc |= own && sh.si[k] >= 4 * g && sh.si[k] < 4 * g + 4 && sh.sj[k] >= max(e0, 0) && sh.sj[k] < min(e0 + R, T.h);
-    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * S::MAIL;
-    const ResSend<S> send(box, T, c, g, e0);
-    const ResRecv<S> recv(T, tid, nt);
+    using Mail = ResMail<S, (CAP > 1)>;
+    const Mail mb(c);
+    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * mb.all;
+    const ResSend<S, Mail> send(box, T, c, mb, g, e0);
+    const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const prow = p00 + e0 * PP + 4 * g;            // p of (e0, g)
     float *const zrow = &sh.vz[e0 + 2 * M][4 * lane];     // v_z of (e0, g)
     const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
@@ -497,7 +531,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
         __syncthreads();
         // ------------------------------------------------------------------ pressure
         const unsigned tag = (unsigned)(n - a.n0) + 1u;
-        const int slot = (n & 1) * S::SLOT;
+        const int slot = (n & 1) * mb.slot;
         if (hrow) hrow += a.slot;
         {
             float4 w[R + HR];   // v_z rows e0 - M .. e0 + R - 1 + M - 1
@@ -525,7 +559,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
                         if (sh.sj[k] == e && e >= 0 && e < T.h && i >= 0 && i < 4)
                             add_source<false>(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
                     }
-            send.put(T, slot, e0, p, tag);
+            send.put(T, mb, slot, e0, p, tag);
             if (own) {
                 if (inner) {
 #pragma unroll
@@ -549,16 +583,16 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 if (e0 + r == 0) v = p[r].x;
-            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(box - (long long)(c.tx + 1) * S::MAIL + 2 * S::SLOT + (n & 3)),
+            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(box - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3)),
                          "l"((unsigned long long)tag << 32 | __float_as_uint(v))
                          : "memory");
         }
-        bool ok = recv.get(box + slot, T, p00, tag, tid, nt);
+        bool ok = recv.get(box + slot, T, mb, p00, tag, tid, nt);
         if (tid == 0 && sh.rec.diag && T.R && T.D) {
             unsigned long long v = 0;
             int spin = 0;
             do {
-                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(box + 2 * S::SLOT + (n & 3)) : "memory");
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(box + 2 * mb.slot + (n & 3)) : "memory");
             } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
             ok = ok && spin < RES_SPIN;
             p00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
@@ -744,9 +778,11 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (own && sh.has[e0 + r + M]) hinj |= 1u << r;
-    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * S::MAIL;
-    const ResSend<S> send(box, T, c, g, e0);
-    const ResRecv<S> recv(T, tid, nt);
+    using Mail = ResMail<S, (CAP > 1)>;
+    const Mail mb(c);
+    unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * mb.all;
+    const ResSend<S, Mail> send(box, T, c, mb, g, e0);
+    const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const qrow = q00 + e0 * PP + 4 * g;
     const float *const prow = p00 + e0 * PP + 4 * g;
     float *const zrow = &sh.bz[e0 + 2 * M][4 * lane];
@@ -825,7 +861,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
         __syncthreads();
         // ------------------------------------------------------------------ pressure
         const unsigned tag = (unsigned)it + 1u;
-        const int slot = (it & 1) * S::SLOT;
+        const int slot = (it & 1) * mb.slot;
         {
             float4 w[R + HR];   // b_z u_z rows e0 - M .. e0 + R - 1 + M - 1
 #pragma unroll
@@ -865,13 +901,13 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
             float4 q[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) q[r] = pmul(rscale(azr[r], axv), pmul(Kv[r], pb[r]));
-            send.put(T, slot, e0, q, tag);
+            send.put(T, mb, slot, e0, q, tag);
             if (own)
 #pragma unroll
                 for (int r = 0; r < R; ++r)
                     if (inner || (e0 + r >= 0 && e0 + r < T.h)) st4(qrow + r * PP, q[r]);
         }
-        if (!recv.get(box + slot, T, q00, tag, tid, nt)) {
+        if (!recv.get(box + slot, T, mb, q00, tag, tid, nt)) {
             *reinterpret_cast<volatile int *>(&sh.abort) = 1;
             atomicOr(stt, ST_ETIMEOUT);
         }
@@ -1013,10 +1049,12 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         hsrc |= own && sh.si[k] >= 4 * g && sh.si[k] < 4 * g + 4 && sh.sj[k] >= max(e0, 0) && sh.sj[k] < min(e0 + R, T.h);
+    using Mail = ResMail<S, (CAP > 1)>;
+    const Mail mb(c);
     const long long tile = (long long)T.s * c.tx * c.tz + T.t;
-    unsigned long long *const boxp = a.mail + tile * S::MAIL, *const boxq = a.mailq + tile * S::MAIL;
-    const ResSend<S> sendp(boxp, T, c, g, e0), sendq(boxq, T, c, g, e0);
-    const ResRecv<S> recv(T, tid, nt);
+    unsigned long long *const boxp = a.mail + tile * mb.all, *const boxq = a.mailq + tile * mb.all;
+    const ResSend<S, Mail> sendp(boxp, T, c, mb, g, e0), sendq(boxq, T, c, mb, g, e0);
+    const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const prow = p00 + e0 * PP + 4 * g, *const qrow = q00 + e0 * PP + 4 * g;
     float *const vrow = &sh.vz[e0 + 2 * M][4 * lane], *const urow = &sh.uz[e0 + 2 * M][4 * lane];
     const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
@@ -1073,7 +1111,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
         __syncthreads();
         // ------------------------------------------------------------------ pressure
         const unsigned tag = (unsigned)(n - a.n0) + 1u;
-        const int slot = (n & 1) * S::SLOT;
+        const int slot = (n & 1) * mb.slot;
         {
             float4 dv[R];
             {
@@ -1125,8 +1163,8 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
                 }
             if (n + 1 < a.n1) wn = __ldg(a.src.wav + n + 1);
         }
-        sendp.put(T, slot, e0, p, tag);
-        sendq.put(T, slot, e0, q, tag);
+        sendp.put(T, mb, slot, e0, p, tag);
+        sendq.put(T, mb, slot, e0, q, tag);
         if (own)
 #pragma unroll
             for (int r = 0; r < R; ++r)
@@ -1140,17 +1178,17 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 if (e0 + r == 0) v = q[r].x;
-            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(boxq - (long long)(c.tx + 1) * S::MAIL + 2 * S::SLOT + (n & 3)),
+            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(boxq - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3)),
                          "l"((unsigned long long)tag << 32 | __float_as_uint(v))
                          : "memory");
         }
-        bool ok = recv.get(boxp + slot, T, p00, tag, tid, nt);
-        ok = recv.get(boxq + slot, T, q00, tag, tid, nt) && ok;
+        bool ok = recv.get(boxp + slot, T, mb, p00, tag, tid, nt);
+        ok = recv.get(boxq + slot, T, mb, q00, tag, tid, nt) && ok;
         if (tid == 0 && sh.rec.diag && T.R && T.D) {
             unsigned long long v = 0;
             int spin = 0;
             do {
-                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(boxq + 2 * S::SLOT + (n & 3)) : "memory");
+                asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(boxq + 2 * mb.slot + (n & 3)) : "memory");
             } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
             ok = ok && spin < RES_SPIN;
             q00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
