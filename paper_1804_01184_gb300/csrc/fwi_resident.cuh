@@ -43,10 +43,15 @@ struct ResShape {
     static constexpr int PZ = 128;                   // pitch of a v_z row: lane l at 4 l
 };
 
-// Four rows a warp (five at 4th order, whose windows are shorter): 96 registers of fields and model a thread and room for the stencil windows
-// (eight rows, 255 registers, 8 warps an SM: 4.9 us a step against 3.4 us; two rows, 20 warps: 3.9 us).
+// Rows a warp, against 12 warps of 168 registers an SM (24 of fields and model a row).  Three leave
+// the windows in registers and give short tiles all 12 warps; four (five at 4th order, whose
+// windows are shorter) make taller tiles, for grids that would not fit and for the engine,
+// whose launches other jobs fill.  Measured (us a step, 8th order): 10 shots of 201^2 2.9 with three
+// rows, 3.2 with four; 16 warps of two 3.4 (their tiles need two launches); 8 warps of eight 4.3.
 using ResFwd2 = ResShape<2, 5, 12>;
+using ResFwd2s = ResShape<2, 3, 12>;
 using ResFwd4 = ResShape<4, 4, 12>;
+using ResFwd4s = ResShape<4, 3, 12>;
 
 // Cut of a shot's grid: tx x tz tiles; the first grem (hrem) tiles have one column group (row)
 // more than gbase (hbase).
@@ -632,8 +637,11 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
 // step nhi's.
 
 constexpr int RES_ENT = 256;    // injection cells of a tile listed in shared memory
+// three rows: 4.8 us a step for 10 shots of 201^2, four 6.0 (the second window spills)
 using ResAdj2 = ResShape<2, 4, 12>;
+using ResAdj2s = ResShape<2, 3, 12>;
 using ResAdj4 = ResShape<4, 4, 12>;
+using ResAdj4s = ResShape<4, 3, 12>;
 
 struct ResAdjArgs {
     const float *ap0, *avx0, *avz0;   // pbar^{nhi+1} (injected), vbar of the launch's shots
@@ -934,7 +942,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
 //
 // Background and scattered wavefields (see k_born_warp) stepped together on chip: the forward
 // kernel's structure with two of everything.  Three rows a warp; the model's perturbation sits in
-// shared memory, read by its own lane alone.
+// shared memory, read by its own lane alone.  10 shots of 201^2: 6.9 us a step (two rows 7.6).
 using ResBorn2 = ResShape<2, 3, 12>;
 using ResBorn4 = ResShape<4, 3, 12>;
 
