@@ -357,6 +357,34 @@ void dyn_smem(const void *kernel, size_t bytes)
         LAUNCH(kernel, grid, block, smem, stream, __VA_ARGS__);    \
     } while (0)
 
+// Launch of a kernel that begins with fwi::step_begin(): its blocks may be placed while the previous
+// kernel's last ones still run.
+template <class... P, class... A>
+cudaError_t launch_step(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+#define PLAUNCH(kernel, grid, block, smem, stream, ...)                          \
+    do {                                                                         \
+        if (smem) dyn_smem((const void *)kernel, smem);                          \
+        cudaEvent_t *ev_ = g_prof.next(#kernel);                                 \
+        if (ev_) cudaEventRecord(ev_[0], stream);                                \
+        launch_step(kernel, grid, block, smem, stream, __VA_ARGS__);             \
+        if (ev_) cudaEventRecord(ev_[1], stream);                                \
+        ++g_launches;                                                            \
+    } while (0)
+
 // Warps of `kernel` (blocks of `threads`, `smem` bytes of dynamic shared memory) resident on
 // the whole GPU at once, from the occupancy calculator; cached per kernel and device.
 int resident_warps(const void *kernel, int threads, size_t smem)
@@ -626,13 +654,13 @@ struct Fwd {
         // queues otherwise take it to 184 registers and 10 resident warps, 6 % slower)
         if (P.M == 2) {
             switch (P.variant) {
-            case 1: SLAUNCH((fwi::k_fwd_warp<2, B128>), grid, T, S, st, args, tl); break;
-            default: SLAUNCH((fwi::k_fwd_warp<2, B170>), grid, T, S, st, args, tl);
+            case 1: PLAUNCH((fwi::k_fwd_warp<2, B128>), grid, T, S, st, args, tl); break;
+            default: PLAUNCH((fwi::k_fwd_warp<2, B170>), grid, T, S, st, args, tl);
             }
         } else {
             switch (P.variant) {
-            case 1: SLAUNCH((fwi::k_fwd_warp<4, B128>), grid, T, S, st, args, tl); break;
-            default: SLAUNCH((fwi::k_fwd_warp<4, B170>), grid, T, S, st, args, tl);
+            case 1: PLAUNCH((fwi::k_fwd_warp<4, B128>), grid, T, S, st, args, tl); break;
+            default: PLAUNCH((fwi::k_fwd_warp<4, B170>), grid, T, S, st, args, tl);
             }
         }
         g_tuner.finish(key, ts, st);
@@ -778,7 +806,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
             const int lo = std::max(n / P.acc * P.acc, n0);
             const float *pl = snap + (size_t)(lo - n0) * slot;
             if (P.nr > 0)
-                LAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[first]),
+                PLAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[first]),
                        at<float>(work, P.accK), snap + (size_t)(n + 1 - n0) * slot, bg, P.nr, P.nt, n, d.Np,
                        at<long long>(work, P.ridx), at<float>(work, P.rw), at<int>(work, P.rl), res);
             int rc = res_adjoint(P, work, st, ra, bg, n, lo, first, pl, res);
@@ -790,7 +818,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
         for (int n = n1 - 1; !chip && n >= n0; --n) {
             const float *pn = snap + (size_t)(n - n0) * slot, *pn1 = snap + (size_t)(n + 1 - n0) * slot;
             if (P.nr > 0)   // pbar^{n+1} += R^T r_n, with its K-gradient term (R^T r_n) p^{n+1}
-                LAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[(n + 1) & 1]),
+                PLAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[(n + 1) & 1]),
                        at<float>(work, P.accK), pn1, bg, P.nr, P.nt, n, d.Np, at<long long>(work, P.ridx),
                        at<float>(work, P.rw), at<int>(work, P.rl), res);
             const size_t S = P.M == 2 ? fwi::adj_smem<2>() : fwi::adj_smem<4>();
@@ -803,15 +831,15 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
             constexpr int B128 = fwi::minb(128, 32), B170 = fwi::minb(170, 32);
             if (P.M == 2) {
                 switch (P.variant) {
-                case 1: SLAUNCH((fwi::k_adj_warp<2, B128>), grid, 32, S, st, args); break;
-                case 2: SLAUNCH((fwi::k_adj_warp<2, B170>), grid, 32, S, st, args); break;
-                default: SLAUNCH((fwi::k_adj_warp<2, 1>), grid, 32, S, st, args);
+                case 1: PLAUNCH((fwi::k_adj_warp<2, B128>), grid, 32, S, st, args); break;
+                case 2: PLAUNCH((fwi::k_adj_warp<2, B170>), grid, 32, S, st, args); break;
+                default: PLAUNCH((fwi::k_adj_warp<2, 1>), grid, 32, S, st, args);
                 }
             } else {
                 switch (P.variant) {
-                case 1: SLAUNCH((fwi::k_adj_warp<4, B128>), grid, 32, S, st, args); break;
-                case 2: SLAUNCH((fwi::k_adj_warp<4, B170>), grid, 32, S, st, args); break;
-                default: SLAUNCH((fwi::k_adj_warp<4, 1>), grid, 32, S, st, args);
+                case 1: PLAUNCH((fwi::k_adj_warp<4, B128>), grid, 32, S, st, args); break;
+                case 2: PLAUNCH((fwi::k_adj_warp<4, B170>), grid, 32, S, st, args); break;
+                default: PLAUNCH((fwi::k_adj_warp<4, 1>), grid, 32, S, st, args);
                 }
             }
             g_tuner.finish(key, ts, st);
@@ -981,11 +1009,11 @@ int fwi_born(const fwi_grid *g, fwi_param pz, const float *xi_a, const float *xi
                   G(P.vz), G(P.dp), G(P.dvx), G(P.dvz), mo, pe, d, P.st, sr, n, tz, bg}
             constexpr int B170 = fwi::minb(170, 32);
             if (P.M == 2) {
-                if (P.variant == 2) SLAUNCH((fwi::k_born_warp<2, B170>), grid, 32, S, st, BORN_ARGS, tl);
-                else SLAUNCH((fwi::k_born_warp<2, 1>), grid, 32, S, st, BORN_ARGS, tl);
+                if (P.variant == 2) PLAUNCH((fwi::k_born_warp<2, B170>), grid, 32, S, st, BORN_ARGS, tl);
+                else PLAUNCH((fwi::k_born_warp<2, 1>), grid, 32, S, st, BORN_ARGS, tl);
             } else {
-                if (P.variant == 2) SLAUNCH((fwi::k_born_warp<4, B170>), grid, 32, S, st, BORN_ARGS, tl);
-                else SLAUNCH((fwi::k_born_warp<4, 1>), grid, 32, S, st, BORN_ARGS, tl);
+                if (P.variant == 2) PLAUNCH((fwi::k_born_warp<4, B170>), grid, 32, S, st, BORN_ARGS, tl);
+                else PLAUNCH((fwi::k_born_warp<4, 1>), grid, 32, S, st, BORN_ARGS, tl);
             }
             g_tuner.finish(key, ts, st);
 #undef BORN_ARGS

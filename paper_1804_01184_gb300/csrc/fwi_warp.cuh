@@ -151,6 +151,16 @@ __device__ __forceinline__ void red_add4(float *dst, float4 v)
                  : "memory");
 }
 
+// Programmatic dependent launch of the time-step kernels: a step's blocks may take the slots that the
+// previous step's last ones leave, and wait here, before their first global access, until that
+// step is complete.  Saves the launch's latency (2 to 4 us a step); without the launch attribute
+// both are no-ops.
+__device__ __forceinline__ void step_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Does the strip hold any source cell of its shot? (uniform per warp)
 __device__ __forceinline__ bool strip_has_src(const SrcCells &sc, int x0, int z0, int zend)
 {
@@ -337,6 +347,7 @@ __global__ void __launch_bounds__(32 * FWD_WPB, MINB) k_fwd_warp(FwdArgs a, Tail
 {
     extern __shared__ __align__(16) unsigned char fwi_smem[];
     const int w = blockIdx.x * FWD_WPB + (threadIdx.x >> 5), nw = strip_warps(a.d, a.tz, a.nshots);
+    step_begin();
     if (w >= nw) {   // a sampling warp
         sample_tail(tl, (w - nw) * 32 + (threadIdx.x & 31));
         return;
@@ -609,6 +620,7 @@ __global__ void __launch_bounds__(32, MINB) k_adj_warp(AdjArgs a)
 {
     extern __shared__ __align__(16) unsigned char fwi_smem[];   // one warp per block
     bool valid;
+    step_begin();
     const Strip sp = strip_of(a.d, a.tz, a.nshots, 1, valid);
     if (!valid) return;
     adj_body<M>(a, sp, *reinterpret_cast<AdjSmem<M> *>(fwi_smem));
@@ -659,6 +671,7 @@ __global__ void k_adj_inject_k(float *__restrict__ ap, float *__restrict__ accK,
                                const float *__restrict__ rw, const int *__restrict__ rl, const float *__restrict__ res)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    step_begin();
     if (t >= ns * 4 * nr) return;
     const int s = t / (4 * nr);
     inject_entry(ap, accK, pn1, s, t - s * 4 * nr, nr, nt, n, Np, ridx, rw, rl, res);
@@ -843,6 +856,7 @@ __global__ void __launch_bounds__(32, MINB) k_born_warp(BornArgs a, Tail tl)
 {
     extern __shared__ __align__(16) unsigned char fwi_smem[];
     const int w = blockIdx.x, nw = strip_warps(a.d, a.tz, a.nshots);
+    step_begin();
     if (w >= nw) {   // a sampling warp
         sample_tail(tl, (w - nw) * 32 + (threadIdx.x & 31));
         return;
