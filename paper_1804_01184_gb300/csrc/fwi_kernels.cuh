@@ -332,8 +332,8 @@ __device__ __forceinline__ double block_sum(double v)
 // misfit of one set of traces (Sec. "Modelling and Inversion"), each trace (nt samples) weighted
 // by w[trace] (w null: 1).  One cluster; its blocks' sums meet in block 0's shared memory in block
 // order.  The FP64 pipe (two lanes an SM) bounds it: a subtraction and a multiply-add an element,
-// half of the total taken at the end, over the cluster's SMs.  1.4 M elements: 1974 us in one block
-// with five FP64 operations an element.
+// half of the total taken at the end, over the cluster's SMs.  1.4 M elements: 106 us (1974 in one
+// block with five FP64 operations an element).
 constexpr int MISFIT_NT = 512;
 
 __global__ void __launch_bounds__(MISFIT_NT) k_misfit(const float *__restrict__ tr, const float *__restrict__ data,
