@@ -28,6 +28,10 @@
  *  - Return value: FWI_OK (0) or a negative FWI_E* code; fwi_last_error() gives a message
  *    (thread-local, valid until the next call on the same thread).
  *  - Work on different streams must use different workspaces.
+ *  - Time steps of grids that fit the GPU's registers run on chip, many steps a launch: a
+ *    cooperative launch, which waits until the whole GPU can hold it, and whose blocks exchange
+ *    their edges through the workspace.  The others stream through memory, a step a launch.
+ *    Results are bitwise the same either way.
  */
 #ifndef FWI_H_
 #define FWI_H_
@@ -153,7 +157,9 @@ int fwi_misfit_weighted(const float *traces, const float *data, long long ntrace
                         double *misfit, void *stream);
 
 /* Waits for `stream` and returns the data-dependent status recorded by the last operation
- * that used `work` (FWI_OK, FWI_EINVAL, FWI_ECFL), then clears it. */
+ * that used `work` (FWI_OK, FWI_EINVAL, FWI_ECFL, or FWI_ETIMEOUT: a block of an on-chip
+ * launch gave up waiting for a neighbour's edge after some seconds, and the results are
+ * undefined), then clears it. */
 int fwi_status(void *work, void *stream);
 
 /* Message for the last error on this thread ("" if none). */
@@ -189,7 +195,7 @@ int fwi_model_noalloc(const fwi_grid *g, fwi_param pz, const float *xi_a, const 
 
 /* fwi_status for fwi_model_noalloc (no counterpart in the paper): waits for `stream` and
  * returns the data-dependent status the last fwi_model_noalloc call on the current device
- * recorded in the built-in scratch (FWI_OK, FWI_EINVAL, FWI_ECFL), then clears it; FWI_OK
+ * recorded in the built-in scratch (the codes of fwi_status), then clears it; FWI_OK
  * when no such call has run on this device.  Allocates nothing. */
 int fwi_status_noalloc(void *stream);
 
@@ -229,8 +235,8 @@ int fwi_set_accumulation(int steps);
  * under stream capture are not timed).  tz > 0 (any number of rows) fixes the height instead,
  * for plans made afterwards by any thread (0 restores tuning); variant picks the register
  * budget per thread of the single-job kernels (0 = default: unbounded, 170 for the forward
- * kernel; 1 = 128; 2 = 170).  Results are
- * bitwise identical for every setting; only speed changes. */
+ * kernel; 1 = 128; 2 = 170).  Either override makes the plans' steps stream also where they
+ * would run on chip.  Results are bitwise identical for every setting; only speed changes. */
 int fwi_set_tile(int tz, int variant);
 
 /* ---------------------------------------------------------------------------------------
@@ -244,7 +250,9 @@ int fwi_set_tile(int tz, int variant);
  * when they finish, so new jobs join while earlier ones still run.
  * fwi_engine_run() advances every admitted job by one time step per iteration; the steps of
  * all running jobs of one kind go out as one batched kernel launch (up to 96 jobs per
- * launch, larger batches split).  Each job computes exactly what the matching single-job
+ * launch, larger batches split).  Jobs whose grids fit take their iterations in runs on chip
+ * instead, as many jobs a launch as the GPU holds at once, so within one call jobs may be
+ * many steps apart.  Each job computes exactly what the matching single-job
  * call (fwi_model, fwi_born, fwi_gradient) computes with a workspace of
  * fwi_workspace_bytes(grid, ns, nr, op, work_budget) bytes: its results are bitwise
  * independent of the other jobs it runs beside.
@@ -359,8 +367,9 @@ size_t fwi_fborn_workspace_bytes(const fwi_fgrid *g, int ns, int nr);
 
 /* Fills the workspace for one acquisition: freqs [nf] (Hz, > 0), spectrum [nf] complex
  * S(w_f), src_xy [ns][2], rec_xy [nr][2] -- HOST arrays, copied before the call returns --
- * and the Green tables of every source and receiver at every node and frequency (double-
- * precision Bessel functions, stored as float pairs).  FWI_EINVAL for a point within dx/2 of
+ * and the Green tables of every source and receiver at every node and frequency (from
+ * double-precision Bessel functions, at the nodes' distances or, for large acquisitions, through
+ * their Taylor expansions between tabulated distances; stored as float pairs).  FWI_EINVAL for a point within dx/2 of
  * a node, a non-positive frequency or bad sizes; FWI_ENOMEM if work_bytes is too small.  The
  * other fwi_fborn_* calls read this workspace with the same (g, ns, nr). */
 int fwi_fborn_tables(const fwi_fgrid *g, const double *freqs, const float *spectrum, const float *src_xy, int ns,
