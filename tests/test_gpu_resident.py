@@ -191,3 +191,36 @@ def test_under_stream_capture(F):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, ref)
+
+
+def test_two_threads_on_two_streams(F):
+    """Cooperative launches that each nearly fill the GPU, from two threads on their own streams."""
+    import threading
+
+    w = case(161, 161, 8, 20, ns=10, nr=20, nt=60)
+    g = gpu_grid(w)
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    ar = (g, w.pz, d(w.xi_a), d(w.xi_b), d(w.src_xy), d(w.wavelet), d(w.rec_xy))
+    ref = F.fwi_model(*ar)
+    torch.cuda.synchronize()
+    out, errors = [[], []], []
+
+    def run(k):
+        try:
+            st, work = torch.cuda.Stream(), F.workspace(g, w.ns, w.nr, F.OP_MODEL)
+            torch.cuda.synchronize()
+            for _ in range(8):
+                with torch.cuda.stream(st):
+                    out[k].append(F.fwi_model(*ar, work=work, check=False))
+            F.fwi_status(work, st)
+        except Exception as e:   # noqa: BLE001 -- shown by the assertion below
+            errors.append(e)
+
+    threads = [threading.Thread(target=run, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    assert all(torch.equal(x, ref) for xs in out for x in xs)
