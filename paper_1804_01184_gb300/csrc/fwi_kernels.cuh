@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace fwi {
 
 struct Dims {
@@ -331,7 +333,8 @@ __device__ __forceinline__ double block_sum(double v)
 // J = 1/2 sum w (tr - data)^2 in FP64 (a fixed summation order, no scratch): the least-squares
 // misfit of one set of traces (Sec. "Modelling and Inversion"), each trace (nt samples) weighted
 // by w[trace] (w null: 1).  One cluster; its blocks' sums meet in block 0's shared memory in block
-// order.  The FP64 pipe (two lanes an SM) bounds it: a subtraction and a multiply-add an element,
+// order (a barrier that every block passes by starting, and waits for after its summation, comes
+// before: another block's shared memory is there only once that block runs).  The FP64 pipe (two lanes an SM) bounds it: a subtraction and a multiply-add an element,
 // half of the total taken at the end, over the cluster's SMs.  1.4 M elements: 106 us (1974 in one
 // block with five FP64 operations an element).
 constexpr int MISFIT_NT = 512;
@@ -343,6 +346,7 @@ __global__ void __launch_bounds__(MISFIT_NT) k_misfit(const float *__restrict__ 
     __shared__ double sh[MISFIT_NT / 32], blocks[16];
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
+    auto started = cl.barrier_arrive();
     const int nb = (int)cl.num_blocks(), b = (int)cl.block_rank();
     const long long step = (long long)nb * MISFIT_NT;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -367,6 +371,7 @@ __global__ void __launch_bounds__(MISFIT_NT) k_misfit(const float *__restrict__ 
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
+    cl.barrier_wait(std::move(started));
     if (threadIdx.x == 0) {
         v = 0.0;
         for (int i = 0; i < MISFIT_NT / 32; ++i) v += sh[i];
