@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "../../include/fwi.h"
+#include "fwi_device.h"
 #include "fwi_kernels.cuh"
 #include "fwi_stream.cuh"
 #include "fwi_warp.cuh"
@@ -1084,6 +1085,27 @@ int fwi_status(void *work, void *stream)
 
 const char *fwi_last_error(void) { return g_err.c_str(); }
 
+// Blocks of k_misfit's one cluster on the current device: 16 where it runs such clusters (the
+// attribute is the device's), 8 (portable) elsewhere.
+static int misfit_width(int)
+{
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute at[1];
+    c.gridDim = dim3(16);
+    c.blockDim = dim3(fwi::MISFIT_NT);
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {16, 1, 1};
+    c.attrs = at;
+    c.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(fwi::k_misfit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, fwi::k_misfit, &c) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+    }
+    return n > 0 ? 16 : 8;
+}
+
 int fwi_misfit_weighted(const float *traces, const float *data, long long ntraces, int nt, const float *weights,
                         double *misfit, void *stream)
 {
@@ -1092,24 +1114,10 @@ int fwi_misfit_weighted(const float *traces, const float *data, long long ntrace
     if (ntraces < 0 || nt < 1 || !misfit || (ntraces > 0 && (!traces || !data)))
         return fail(FWI_EINVAL, "invalid misfit arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // one cluster: 16 blocks where the device runs such clusters, 8 (portable) elsewhere
-    static const int wide = [] {
-        cudaLaunchConfig_t c = {};
-        cudaLaunchAttribute at[1];
-        c.gridDim = dim3(16);
-        c.blockDim = dim3(fwi::MISFIT_NT);
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim = {16, 1, 1};
-        c.attrs = at;
-        c.numAttrs = 1;
-        int n = 0;
-        if (cudaFuncSetAttribute(fwi::k_misfit, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, fwi::k_misfit, &c) != cudaSuccess) {
-            cudaGetLastError();
-            n = 0;
-        }
-        return n > 0 ? 16 : 8;
-    }();
+    int dev = 0;
+    CK(cudaGetDevice(&dev));
+    static fwi::PerDevice<int> widths;
+    const int wide = widths.get(dev, misfit_width);
     const long long n = ntraces * nt;
     // small sums: no more blocks than there are four elements a thread for
     unsigned nb = 1;
