@@ -55,6 +55,8 @@ CASES = {
     # distances that are whole intervals (h = 1): both sides of an interval's edge and of the first one
     "interval edges": dict(nx=200, nz=40, dx=1.0, x0=0.0, z0=0.0, src=np.array([[-3.0, 0.0], [-40.0, 5.0]], np.float32),
                            rec=np.array([[203.0, 0.0], [-64.0, 3.0], [-63.0, 7.0], [230.0, 39.0]], np.float32), f=0.5 * np.arange(1, 31), radial=1, near=1),
+    # wavenumbers whose pairs FP32 does not hold
+    "seven decades of frequency": dict(nx=60, nz=41, dx=5.0, src=ring(2, 195.0), rec=ring(8, 195.0, 0.5), f=np.geomspace(1e-6, 13.0, 33), radial=0, near=1),
     "every node near": dict(nx=40, nz=40, dx=5.0, src=ring(2, 160.0), rec=ring(6, 160.0, 0.5), f=0.01 * np.arange(1, 3), radial=0, near=1),
     "too small to pay": dict(nx=200, nz=3, dx=2.0, src=ring(1, 230.0), rec=ring(2, 230.0, 0.5), f=0.5 * np.arange(1, 33), radial=0, near=1),
 }
