@@ -303,7 +303,7 @@ __global__ void k_sample(const float *__restrict__ p, int ns, int nr, int nt, in
     float v = 0.f;
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-        if (FWI_IN(true, ridx[4 * r + c], 1, Np, nullptr)) v += rw[4 * r + c] * ps[ridx[4 * r + c]];
+        if (FWI_IN(true, ridx[4 * r + c], 1, Np, nullptr)) v = fmaf(rw[4 * r + c], ps[ridx[4 * r + c]], v);
     traces[(long long)t * nt + n] = v;
 }
 

@@ -284,10 +284,10 @@ __device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, c
         for (int k = tid; k < rc.n; k += blockDim.x) {
             const float *q = p + rc.off[k];
             float v = 0.f;
-            v += rc.w[k][0] * q[0];
-            v += rc.w[k][1] * q[1];
-            v += rc.w[k][2] * q[PP];
-            v += rc.w[k][3] * q[PP + 1];
+            v = fmaf(rc.w[k][0], q[0], v);
+            v = fmaf(rc.w[k][1], q[1], v);
+            v = fmaf(rc.w[k][2], q[PP], v);
+            v = fmaf(rc.w[k][3], q[PP + 1], v);
             traces[((long long)T.s * nr + rc.r[k]) * nt + n] = v;
         }
         return;
@@ -298,10 +298,10 @@ __device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, c
         if (j < 0 || j >= T.h || i < 0 || i >= 4 * T.ng) continue;
         const float *q = p + j * PP + i;
         float v = 0.f;
-        v += rw[4 * k] * q[0];
-        v += rw[4 * k + 1] * q[1];
-        v += rw[4 * k + 2] * q[PP];
-        v += rw[4 * k + 3] * q[PP + 1];
+        v = fmaf(rw[4 * k], q[0], v);
+        v = fmaf(rw[4 * k + 1], q[1], v);
+        v = fmaf(rw[4 * k + 2], q[PP], v);
+        v = fmaf(rw[4 * k + 3], q[PP + 1], v);
         traces[((long long)T.s * nr + k) * nt + n] = v;
     }
 }
@@ -411,18 +411,6 @@ __device__ __forceinline__ void warp_sides(const float4 &b, float4 &l, float4 &r
     r.x = __shfl_down_sync(all, b.x, 1);
     if (M > 2) r.y = __shfl_down_sync(all, b.y, 1);
     if (M > 3) r.z = __shfl_down_sync(all, b.z, 1);
-}
-
-// Component i of v += kw * w: with product and sum rounded apart, or together (FUSED).  Which, is what
-// the compiler made of the streaming kernels' injection, whose results these kernels reproduce.
-template <bool FUSED>
-__device__ __forceinline__ void add_source(float4 &v, int i, float kw, float w)
-{
-    auto add = [&](float x) { return FUSED ? fmaf(kw, w, x) : __fadd_rn(x, __fmul_rn(kw, w)); };
-    v.x = i == 0 ? add(v.x) : v.x;
-    v.y = i == 1 ? add(v.y) : v.y;
-    v.z = i == 2 ? add(v.z) : v.z;
-    v.w = i == 3 ? add(v.w) : v.w;
 }
 
 // Forward steps n0 .. n1 - 1.

@@ -64,9 +64,18 @@ __device__ __forceinline__ float4 operator*(float4 a, float4 b) { return make_fl
 __device__ __forceinline__ float4 operator*(float s, float4 b) { return make_float4(s * b.x, s * b.y, s * b.z, s * b.w); }
 __device__ __forceinline__ float4 fma4(float s, float4 a, float4 c) { return make_float4(fmaf(s, a.x, c.x), fmaf(s, a.y, c.y), fmaf(s, a.z, c.z), fmaf(s, a.w, c.w)); }
 __device__ __forceinline__ float comp(const float4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
-__device__ __forceinline__ void addc(float4 &v, int k, float a)
+// Component i of v += kw * w, a source's injection.  Product and sum are rounded apart, or together
+// (FUSED): the forward steps use the former and the Born steps the latter, streaming and on chip.
+// Explicit, like every operation that both kinds of kernel share, because their results are to be
+// bitwise the same whatever the compiler would contract.
+template <bool FUSED>
+__device__ __forceinline__ void add_source(float4 &v, int i, float kw, float w)
 {
-    if (k == 0) v.x += a; else if (k == 1) v.y += a; else if (k == 2) v.z += a; else v.w += a;
+    auto add = [&](float x) { return FUSED ? fmaf(kw, w, x) : __fadd_rn(x, __fmul_rn(kw, w)); };
+    v.x = i == 0 ? add(v.x) : v.x;
+    v.y = i == 1 ? add(v.y) : v.y;
+    v.z = i == 2 ? add(v.z) : v.z;
+    v.w = i == 3 ? add(v.w) : v.w;
 }
 // zero the components at columns >= Nx (c0 = first column of the float4)
 __device__ __forceinline__ float4 mask4(float4 v, int c0, int Nx)

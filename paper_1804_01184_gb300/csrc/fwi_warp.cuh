@@ -194,7 +194,7 @@ __device__ __forceinline__ void sample_tail(const Tail &tl, int t)
     float v = 0.f;
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-        if (FWI_IN(true, tl.ridx[4 * r + c], 1, tl.Np, nullptr)) v += tl.rw[4 * r + c] * ps[tl.ridx[4 * r + c]];
+        if (FWI_IN(true, tl.ridx[4 * r + c], 1, tl.Np, nullptr)) v = fmaf(tl.rw[4 * r + c], ps[tl.ridx[4 * r + c]], v);
     tl.traces[(long long)t * tl.nt + tl.col] = v;
 }
 
@@ -328,7 +328,7 @@ __device__ __forceinline__ void fwd_body(const FwdArgs &a, const Strip &sp, FwdS
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     if (sc.j[k] == j && sc.i[k] >= L.mc && sc.i[k] < L.mc + 4)
-                        addc(pn, sc.i[k] - L.mc, comp(Kv, sc.i[k] - L.mc) * wn * sc.w[k]);
+                        add_source<false>(pn, sc.i[k] - L.mc, __fmul_rn(comp(Kv, sc.i[k] - L.mc), wn), sc.w[k]);
             }
             st4(P1 + j * d.Px + L.mc, pn);
         }
@@ -410,7 +410,7 @@ __device__ __forceinline__ void small_work(const SmallTable &s, int u)
         float v = 0.f;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            if (FWI_IN(true, d.ridx[4 * r + c], 1, d.Np, nullptr)) v += d.rw[4 * r + c] * ps[d.ridx[4 * r + c]];
+            if (FWI_IN(true, d.ridx[4 * r + c], 1, d.Np, nullptr)) v = fmaf(d.rw[4 * r + c], ps[d.ridx[4 * r + c]], v);
         d.traces[(long long)l * d.nt + d.n] = v;
         return;
     }
@@ -656,12 +656,12 @@ __device__ __forceinline__ void inject_entry(float *__restrict__ ap, float *__re
     int m = rl[k];
     if (!(m & CHAIN_FIRST)) return;
     const float *rs = res + (long long)s * nr * nt + n;
-    float a = rw[k] * rs[(long long)(k >> 2) * nt];
-    for (m &= CHAIN_FIRST - 1; m < n4; m = rl[m] & (CHAIN_FIRST - 1)) a += rw[m] * rs[(long long)(m >> 2) * nt];
+    float a = __fmul_rn(rw[k], rs[(long long)(k >> 2) * nt]);
+    for (m &= CHAIN_FIRST - 1; m < n4; m = rl[m] & (CHAIN_FIRST - 1)) a = fmaf(rw[m], rs[(long long)(m >> 2) * nt], a);
     if (!FWI_IN(true, ridx[k], 1, Np, nullptr)) return;
     const long long o = (long long)s * Np + ridx[k];
-    ap[o] += a;
-    accK[o] += a * pn1[o];
+    ap[o] = __fadd_rn(ap[o], a);
+    accK[o] = fmaf(a, pn1[o], accK[o]);
 }
 
 // Adds the residual R^T r_n into pbar^{n+1} and the receiver-cell term (R^T r_n) p^{n+1}
@@ -838,8 +838,8 @@ __device__ __forceinline__ void born_body(const BornArgs &a, const Strip &sp, Bo
                 for (int k = 0; k < 4; ++k)
                     if (sc.j[k] == j && sc.i[k] >= L.mc && sc.i[k] < L.mc + 4) {
                         const int c = sc.i[k] - L.mc;
-                        addc(pn, c, comp(K, c) * wn * sc.w[k]);
-                        addc(qn, c, comp(dK, c) * wn * sc.w[k]);
+                        add_source<true>(pn, c, __fmul_rn(comp(K, c), wn), sc.w[k]);
+                        add_source<true>(qn, c, __fmul_rn(comp(dK, c), wn), sc.w[k]);
                     }
             }
             st4(P1 + j * d.Px + L.mc, pn);
