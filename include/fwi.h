@@ -46,7 +46,8 @@ extern "C" {
 #define FWI_EINVAL   -1   /* bad size, null pointer, 1 + xi <= 0, position off the grid */
 #define FWI_ECFL     -2   /* dt above the stability limit of the stencil for the model */
 #define FWI_ENOMEM   -3   /* workspace smaller than the operation's minimum             */
-#define FWI_ETIMEOUT -4   /* a bounded device-side wait expired (fwi_fborn_status) */
+#define FWI_ETIMEOUT -4   /* a bounded device-side wait expired (fwi_status, fwi_engine_run,
+                             fwi_fborn_status)                                           */
 #define FWI_ECUDA    -5   /* a CUDA runtime call failed                                 */
 
 /* Parameterizations of Table 1; contrasts xi = (m - m_o)/m_o of the named pair. */
@@ -227,6 +228,14 @@ int fwi_trace_report(char *buf, size_t len);
  * FWI_EINVAL for steps < 0. */
 int fwi_set_accumulation(int steps);
 
+/* Failure detection of the on-chip time steps (no counterpart in the paper): a block polls for a
+ * neighbour's edge at most `polls` times (about a microsecond each), then gives up, records
+ * FWI_ETIMEOUT (fwi_status, fwi_engine_run) and ends with its launch.  Holds for the launches that
+ * the calling thread enqueues afterwards; a negative value restores the default (2^21, some
+ * seconds).  0 expires at the first step of every launch whose shots span several blocks: the
+ * way to test a caller's handling of the error. */
+int fwi_set_wait_limit(int polls);
+
 /* Launch-shape tuning (no counterpart in the paper: the tile-shape autotuner's hook).  By
  * default the strip height of the streaming kernels is tuned online: for each launch shape
  * the first launches try the height an occupancy rule picks (strips that just fill the warps
@@ -298,7 +307,8 @@ int fwi_engine_submit(fwi_engine *engine, const fwi_job *job, long long *ticket)
  * for the GPU to finish the work of the call before the previous one, so the host never
  * runs more than one call's iterations ahead of the GPU (what bounds the wait of a job
  * submitted between calls).  Returns FWI_OK or the first failure (FWI_ECUDA, ...) of the work
- * it enqueued; after a failure the engine's jobs are undefined: destroy it. */
+ * it enqueued, or FWI_ETIMEOUT, instead of any further ticket, once a bounded wait of an on-chip
+ * launch has expired; after a failure the engine's jobs are undefined: destroy it. */
 int fwi_engine_run(fwi_engine *engine, int iterations, long long *done, int max_done, int *ndone);
 
 /* Cancels a job that is queued or running (a request the caller no longer wants; no

@@ -1175,6 +1175,13 @@ int fwi_trace_report(char *buf, size_t len)
     return (int)out.size();
 }
 
+int fwi_set_wait_limit(int polls)
+{
+    g_err.clear();
+    g_polls = polls < 0 ? fwi::RES_POLLS : polls;
+    return FWI_OK;
+}
+
 int fwi_set_accumulation(int steps)
 {
     if (steps < 0) return fail(FWI_EINVAL, "accumulation chunk must be >= 0 steps");

@@ -28,9 +28,25 @@
 namespace fwi {
 
 constexpr int RES_RC = 64;      // receivers of a tile listed in shared memory
-// a wait gives up after this many polls (a poll is an L2 round trip, ~1 us: a few seconds)
-constexpr int RES_SPIN = 1 << 21;
+// a wait gives up after this many polls unless told otherwise (a poll is an L2 round trip, ~1 us: a
+// few seconds)
+constexpr int RES_POLLS = 1 << 21;
 enum : int { ST_ETIMEOUT = 16 };
+
+// How long a launch's waits last, and where an expired one is recorded besides the operation's status
+// word (the engine's word in host memory, or null).
+struct ResWait {
+    int polls;
+    int *expired;
+};
+
+// A wait of this block has expired.
+__device__ __forceinline__ void res_expired(const ResWait &w, int *status, int *abort)
+{
+    *reinterpret_cast<volatile int *>(abort) = 1;
+    atomicOr(status, ST_ETIMEOUT);
+    if (w.expired) *reinterpret_cast<volatile int *>(w.expired) = 1;
+}
 
 // Shape of a resident CTA: up to NW warps of R rows of 30 column groups.
 template <int M_, int R_, int NW_>
@@ -143,6 +159,7 @@ struct ResFwdArgs {
     int nr, nt;
     int n0, n1;
     ResCut cut;
+    ResWait wait;
     unsigned long long *mail;       // [shots][tiles] mailboxes (ResMail), cleared before the launch
 };
 
@@ -335,9 +352,9 @@ struct ResRecv {
         }
     }
     // words of step `tag` of this tile's mailbox slot m into the halo of the field whose own cell
-    // (0, 0) is at p; false when a wait expired
+    // (0, 0) is at p; false when a wait expired (a limit of 0 expires wherever the tile has neighbours)
     __device__ __forceinline__ bool get(const unsigned long long *m, const ResTile &T, const Mail &B, float *p,
-                                        unsigned tag, int tid, int nt) const
+                                        unsigned tag, int tid, int nt, int polls) const
     {
         int spin = 0;
         if (tid < n) {
@@ -345,21 +362,21 @@ struct ResRecv {
             MailWord4 a, b;
             mail_get4(m + w0, a);
             if (two) mail_get4(m + w1, b);
-            while (!mail_ready(a, tag) && ++spin < RES_SPIN) mail_get4(m + w0, a);
+            while (!mail_ready(a, tag) && ++spin < polls) mail_get4(m + w0, a);
             st4(p + o0, mail_value(a));
             if (two) {
-                while (!mail_ready(b, tag) && ++spin < RES_SPIN) mail_get4(m + w1, b);
+                while (!mail_ready(b, tag) && ++spin < polls) mail_get4(m + w1, b);
                 st4(p + o1, mail_value(b));
             }
             for (int k = tid + 2 * nt; k < n; k += nt) {
                 int w, o;
                 item(T, B, k, w, o);
                 mail_get4(m + w, a);
-                while (!mail_ready(a, tag) && ++spin < RES_SPIN) mail_get4(m + w, a);
+                while (!mail_ready(a, tag) && ++spin < polls) mail_get4(m + w, a);
                 st4(p + o, mail_value(a));
             }
         }
-        return spin < RES_SPIN;
+        return spin < polls || n == 0;
     }
 };
 
@@ -580,20 +597,17 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
                          "l"((unsigned long long)tag << 32 | __float_as_uint(v))
                          : "memory");
         }
-        bool ok = recv.get(box + slot, T, mb, p00, tag, tid, nt);
+        bool ok = recv.get(box + slot, T, mb, p00, tag, tid, nt, a.wait.polls);
         if (tid == 0 && sh.rec.diag && T.R && T.D) {
             unsigned long long v = 0;
             int spin = 0;
             do {
                 asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(box + 2 * mb.slot + (n & 3)) : "memory");
-            } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
-            ok = ok && spin < RES_SPIN;
+            } while ((unsigned)(v >> 32) != tag && ++spin < a.wait.polls);
+            ok = ok && spin < a.wait.polls;
             p00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
         }
-        if (!ok) {
-            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
-            atomicOr(stt, ST_ETIMEOUT);
-        }
+        if (!ok) res_expired(a.wait, stt, &sh.abort);
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
         if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, p00, PP, tid);
@@ -648,6 +662,7 @@ struct ResAdjArgs {
     int nr, nt;
     int nhi, nlo;
     ResCut cut;
+    ResWait wait;
     unsigned long long *mail;
 };
 
@@ -903,10 +918,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
                 for (int r = 0; r < R; ++r)
                     if (inner || (e0 + r >= 0 && e0 + r < T.h)) st4(qrow + r * PP, q[r]);
         }
-        if (!recv.get(box + slot, T, mb, q00, tag, tid, nt)) {
-            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
-            atomicOr(stt, ST_ETIMEOUT);
-        }
+        if (!recv.get(box + slot, T, mb, q00, tag, tid, nt, a.wait.polls)) res_expired(a.wait, stt, &sh.abort);
         cp_wait<0>();
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
@@ -949,6 +961,7 @@ struct ResBornArgs {
     int nr, nt;
     int n0, n1;
     ResCut cut;
+    ResWait wait;
     unsigned long long *mail, *mailq;               // p's and q's mailboxes
 };
 
@@ -1178,21 +1191,18 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
                          "l"((unsigned long long)tag << 32 | __float_as_uint(v))
                          : "memory");
         }
-        bool ok = recv.get(boxp + slot, T, mb, p00, tag, tid, nt);
-        ok = recv.get(boxq + slot, T, mb, q00, tag, tid, nt) && ok;
+        bool ok = recv.get(boxp + slot, T, mb, p00, tag, tid, nt, a.wait.polls);
+        ok = recv.get(boxq + slot, T, mb, q00, tag, tid, nt, a.wait.polls) && ok;
         if (tid == 0 && sh.rec.diag && T.R && T.D) {
             unsigned long long v = 0;
             int spin = 0;
             do {
                 asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(boxq + 2 * mb.slot + (n & 3)) : "memory");
-            } while ((unsigned)(v >> 32) != tag && ++spin < RES_SPIN);
-            ok = ok && spin < RES_SPIN;
+            } while ((unsigned)(v >> 32) != tag && ++spin < a.wait.polls);
+            ok = ok && spin < a.wait.polls;
             q00[T.h * PP + 4 * T.ng] = __uint_as_float((unsigned)v);
         }
-        if (!ok) {
-            *reinterpret_cast<volatile int *>(&sh.abort) = 1;
-            atomicOr(stt, ST_ETIMEOUT);
-        }
+        if (!ok) res_expired(a.wait, stt, &sh.abort);
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
         if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, q00, PP, tid);

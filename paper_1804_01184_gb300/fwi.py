@@ -5,7 +5,7 @@ PyTorch supplies device memory (inputs, outputs and the scratch workspace) and s
 The functions carry the C names: ``fwi_model``, ``fwi_born``, ``fwi_adjoint``,
 ``fwi_gradient`` (optionally weighted per trace), ``fwi_misfit``, ``fwi_workspace_bytes``,
 ``fwi_status``, ``fwi_model_noalloc``, ``fwi_status_noalloc``, ``fwi_set_tile``, ``fwi_set_checkpoint``,
-``fwi_set_accumulation``, ``fwi_trace``.
+``fwi_set_accumulation``, ``fwi_set_wait_limit``, ``fwi_trace``.
 
 There is no fallback: if libfwi.so has not been built (``paper_1804_01184_gb300.build``)
 or no CUDA device is present, these functions raise.
@@ -80,6 +80,7 @@ def _open(path):
     L.fwi_set_tile.argtypes = [C.c_int, C.c_int]
     L.fwi_set_checkpoint.argtypes = [C.c_int]
     L.fwi_set_accumulation.argtypes = [C.c_int]
+    L.fwi_set_wait_limit.argtypes = [C.c_int]
     L.fwi_trace.argtypes = [C.c_int]
     L.fwi_trace_report.argtypes = [C.c_char_p, C.c_size_t]
     L.fwi_model_noalloc.argtypes = [gp, C.c_int, vp, vp, sp, rp, vp, vp]
@@ -200,6 +201,12 @@ def fwi_set_checkpoint(every: int = 0):
 def fwi_set_accumulation(steps: int = 0):
     """Adjoint steps per FP32 gradient-accumulation chunk for plans made afterwards (0 = 64)."""
     _raise(lib().fwi_set_accumulation(int(steps)))
+
+
+def fwi_set_wait_limit(polls: int = -1):
+    """Polls after which a block of an on-chip launch gives up on a neighbour, for the launches
+    this thread enqueues afterwards (negative: the default; 0: at once, to test error handling)."""
+    _raise(lib().fwi_set_wait_limit(int(polls)))
 
 
 def fwi_trace(enable: bool = True):
