@@ -41,7 +41,9 @@ enum : int { ST_EINVAL = 1, ST_ECFL = 2, ST_EBOUNDS = 8 };
 // Checked builds (-DFWI_CHECKED, the debug build): every global load and store of the time-step
 // kernels first tests its offset against the size of its field; a failing test sets
 // ST_EBOUNDS in the operation's status word and the access is skipped (nothing traps), and
-// fwi_status() reports it.  In the default build the tests compile away.
+// fwi_status() reports it.  The on-chip kernels also test their mailbox words against the shot's
+// mailboxes and, once a launch, the rows of shared memory that a thread reads and writes
+// (FWI_SPAN: floats lo .. hi - 1 of an array).  In the default build the tests compile away.
 #ifdef FWI_CHECKED
 __device__ __forceinline__ bool in_field(long long off, long long len, long long lim, int *status)
 {
@@ -50,8 +52,11 @@ __device__ __forceinline__ bool in_field(long long off, long long len, long long
     return false;
 }
 #define FWI_IN(valid, off, len, lim, status) ((valid) && ::fwi::in_field((off), (len), (lim), (status)))
+#define FWI_SPAN(array, lo, hi, status) \
+    ::fwi::in_field((lo) - reinterpret_cast<const float *>(&(array)), (hi) - (lo), sizeof(array) / sizeof(float), (status))
 #else
 #define FWI_IN(valid, off, len, lim, status) (valid)
+#define FWI_SPAN(array, lo, hi, status) true
 #endif
 
 __device__ __forceinline__ long long cell(const Dims &d, int i, int j) { return (long long)j * d.Px + i; }

@@ -229,6 +229,20 @@ __device__ __forceinline__ float4 mail_value(const MailWord4 &r)
                        __uint_as_float((unsigned)r.w[2]), __uint_as_float((unsigned)r.w[3]));
 }
 
+// The mailboxes that a tile may touch, for the checked builds: its shot's.
+struct MailSpan {
+#ifdef FWI_CHECKED
+    const unsigned long long *base;
+    long long words;
+    int *status;
+    __device__ MailSpan(const unsigned long long *b, long long w, int *s) : base(b), words(w), status(s) {}
+    __device__ __forceinline__ bool has(const unsigned long long *m, int len) const { return in_field(m - base, len, words, status); }
+#else
+    __device__ MailSpan(const unsigned long long *, long long, int *) {}
+    __device__ __forceinline__ bool has(const unsigned long long *, int) const { return true; }
+#endif
+};
+
 // This CTA's tile.
 struct ResTile {
     int t, s;            // tile of its shot, shot of the launch
@@ -276,13 +290,14 @@ struct __align__(16) ResFwdSmem {
 };
 
 // The tile's receivers (order irrelevant: each writes its own trace); offsets for pitch PP.
+// lim: floats from own cell (0, 0) to the end of the field (checked builds)
 __device__ __forceinline__ void res_receivers(ResRec &rc, const ResTile &T, const Dims &d, const long long *ridx,
-                                              const float *rw, int nr, int PP, int tid)
+                                              const float *rw, int nr, int PP, int tid, int lim, int *stt)
 {
     for (int k = tid; k < nr; k += blockDim.x) {
         const long long o = ridx[4 * k];
         const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
-        if (j < 0 || j >= T.h || i < 0 || i >= 4 * T.ng) continue;
+        if (!FWI_IN(j >= 0 && j < T.h && i >= 0 && i < 4 * T.ng, j * PP + i, PP + 2, lim, stt)) continue;
         if (j == T.h - 1 && i == 4 * T.ng - 1) rc.diag = 1;
         const int e = atomicAdd(&rc.n, 1);
         if (e >= RES_RC) continue;
@@ -292,10 +307,10 @@ __device__ __forceinline__ void res_receivers(ResRec &rc, const ResTile &T, cons
     }
 }
 
-// trace[s][r][n] of the tile's receivers from p^{n+1} (own cells and halo); `p`: own cell (0, 0)
+// trace[s][r][n] of the tile's receivers from p^{n+1} (own cells and halo); `p`: own cell (0, 0), lim as above
 __device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, const Dims &d, const long long *ridx,
                                            const float *rw, float *traces, int nr, int nt, int n, const float *p, int PP,
-                                           int tid)
+                                           int tid, int lim, int *stt)
 {
     if (rc.n <= RES_RC) {
         for (int k = tid; k < rc.n; k += blockDim.x) {
@@ -312,7 +327,7 @@ __device__ __forceinline__ void res_sample(const ResRec &rc, const ResTile &T, c
     for (int k = tid; k < nr; k += blockDim.x) {
         const long long o = ridx[4 * k];
         const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
-        if (j < 0 || j >= T.h || i < 0 || i >= 4 * T.ng) continue;
+        if (!FWI_IN(j >= 0 && j < T.h && i >= 0 && i < 4 * T.ng, j * PP + i, PP + 2, lim, stt)) continue;
         const float *q = p + j * PP + i;
         float v = 0.f;
         v = fmaf(rw[4 * k], q[0], v);
@@ -354,11 +369,11 @@ struct ResRecv {
     // words of step `tag` of this tile's mailbox slot m into the halo of the field whose own cell
     // (0, 0) is at p; false when a wait expired (a limit of 0 expires wherever the tile has neighbours)
     __device__ __forceinline__ bool get(const unsigned long long *m, const ResTile &T, const Mail &B, float *p,
-                                        unsigned tag, int tid, int nt, int polls) const
+                                        unsigned tag, int tid, int nt, int polls, const MailSpan &box) const
     {
         int spin = 0;
-        if (tid < n) {
-            const bool two = tid + nt < n;
+        if (tid < n && box.has(m + w0, 4)) {
+            const bool two = tid + nt < n && box.has(m + w1, 4);
             MailWord4 a, b;
             mail_get4(m + w0, a);
             if (two) mail_get4(m + w1, b);
@@ -371,6 +386,7 @@ struct ResRecv {
             for (int k = tid + 2 * nt; k < n; k += nt) {
                 int w, o;
                 item(T, B, k, w, o);
+                if (!box.has(m + w, 4)) continue;
                 mail_get4(m + w, a);
                 while (!mail_ready(a, tag) && ++spin < polls) mail_get4(m + w, a);
                 st4(p + o, mail_value(a));
@@ -397,21 +413,24 @@ struct ResSend {
         lr = own && T.L && g < 2 ? box - B.all + B.right + 4 * g
              : own && T.R && g >= T.ng - 2 ? box + B.all + B.left + 4 * (g - (T.ng - 2)) : nullptr;
     }
-    __device__ __forceinline__ void put(const ResTile &T, const Mail &B, int slot, int e0, const float4 (&v)[S::R], unsigned tag) const
+    __device__ __forceinline__ void put(const ResTile &T, const Mail &B, int slot, int e0, const float4 (&v)[S::R], unsigned tag,
+                                        const MailSpan &shot) const
     {
         constexpr int R = S::R;
         if (lr)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (e0 + r >= 0 && e0 + r < T.h) mail_put4(lr + slot + (e0 + r) * 8, v[r], tag);
+                if (e0 + r >= 0 && e0 + r < T.h && shot.has(lr + slot + (e0 + r) * 8, 4)) mail_put4(lr + slot + (e0 + r) * 8, v[r], tag);
         if (up)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (e0 + r >= 0 && e0 + r < S::HR) mail_put4(ud + slot + (e0 + r) * B.w, v[r], tag);
+                if (e0 + r >= 0 && e0 + r < S::HR && shot.has(ud + slot + (e0 + r) * B.w, 4))
+                    mail_put4(ud + slot + (e0 + r) * B.w, v[r], tag);
         if (down)
 #pragma unroll
             for (int r = 0; r < R; ++r)
-                if (e0 + r >= T.h - S::HR && e0 + r < T.h) mail_put4(ud + dn + slot + (e0 + r) * B.w, v[r], tag);
+                if (e0 + r >= T.h - S::HR && e0 + r < T.h && shot.has(ud + dn + slot + (e0 + r) * B.w, 4))
+                    mail_put4(ud + dn + slot + (e0 + r) * B.w, v[r], tag);
     }
 };
 
@@ -462,7 +481,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
         sh.si[tid] = (int)(o % d.Px) - 4 * T.g0;
         sh.sw[tid] = a.src.w[4 * T.s + tid];
     }
-    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid);
+    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid, S::E * PP - 8, stt);
     float *const p00 = &sh.p[HR][8];                      // own cell (0, 0)
     if (a.p0)   // initial pressure of the tile and its halo
         for (int k = tid; k < (T.h + 2 * HR) * (T.ng + 4); k += nt) {
@@ -504,6 +523,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
     using Mail = ResMail<S, (CAP > 1)>;
     const Mail mb(c);
     unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * mb.all;
+    const MailSpan shot(box - (long long)T.t * mb.all, (long long)c.tx * c.tz * mb.all, stt), mine(box, mb.all, stt);
     const ResSend<S, Mail> send(box, T, c, mb, g, e0);
     const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const prow = p00 + e0 * PP + 4 * g;            // p of (e0, g)
@@ -511,6 +531,16 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
     const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
     float *hrow = a.hist ? a.hist + so + go : nullptr;
     const float2 *const nc = a.st.nc;
+#ifdef FWI_CHECKED
+    bool sound = FWI_SPAN(sh.p, prow - (M - 1) * PP - 4, prow + (R - 1 + M) * PP + 8, stt) &&
+                 FWI_SPAN(sh.vz, zrow - M * PZ, zrow + (R + M - 2) * PZ + 4, stt) && in_field(e0 + M, R, S::E, stt);
+    for (int k = tid; k < recv.n; k += nt) {
+        int w, o;
+        recv.item(T, mb, k, w, o);
+        sound = FWI_SPAN(sh.p, p00 + o, p00 + o + 4, stt) && sound;
+    }
+    if (__syncthreads_or(!sound)) return;   // (the neighbours' waits for this tile expire)
+#endif
 
     const bool inner = e0 >= 0 && e0 + R <= T.h;          // every row of the warp is an own row
     float wn = hsrc ? __ldg(a.src.wav + a.n0) : 0.f;
@@ -569,7 +599,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
                         if (sh.sj[k] == e && e >= 0 && e < T.h && i >= 0 && i < 4)
                             add_source<false>(p[r], i, __fmul_rn(comp(Kv[r], i), wn), sh.sw[k]);
                     }
-            send.put(T, mb, slot, e0, p, tag);
+            send.put(T, mb, slot, e0, p, tag, shot);
             if (own) {
                 if (inner) {
 #pragma unroll
@@ -593,12 +623,13 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 if (e0 + r == 0) v = p[r].x;
-            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(box - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3)),
-                         "l"((unsigned long long)tag << 32 | __float_as_uint(v))
-                         : "memory");
+            unsigned long long *const dg = box - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3);
+            if (shot.has(dg, 1))
+                asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(dg), "l"((unsigned long long)tag << 32 | __float_as_uint(v))
+                             : "memory");
         }
-        bool ok = recv.get(box + slot, T, mb, p00, tag, tid, nt, a.wait.polls);
-        if (tid == 0 && sh.rec.diag && T.R && T.D) {
+        bool ok = recv.get(box + slot, T, mb, p00, tag, tid, nt, a.wait.polls, mine);
+        if (tid == 0 && sh.rec.diag && T.R && T.D && mine.has(box + 2 * mb.slot + (n & 3), 1)) {
             unsigned long long v = 0;
             int spin = 0;
             do {
@@ -610,7 +641,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_fwd(const __grid_constant
         if (!ok) res_expired(a.wait, stt, &sh.abort);
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
-        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, p00, PP, tid);
+        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, p00, PP, tid, S::E * PP - 8, stt);
         // the halo's pressure: the groups beside the tile, and the rows above and below it
         if (!own || !inner)
 #pragma unroll
@@ -721,7 +752,8 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
         if (!(a.rl[k] & CHAIN_FIRST)) return -1;
         const long long o = a.ridx[k];
         const int j = (int)(o / d.Px) - T.z0, i = (int)(o % d.Px) - 4 * T.g0;
-        return j >= 0 && j < T.h && i >= 0 && i < 4 * T.ng ? (j + M) * 128 + 4 + i : -1;
+        const int at = (j + M) * 128 + 4 + i;
+        return FWI_IN(j >= 0 && j < T.h && i >= 0 && i < 4 * T.ng, at, 1, S::E * 128, stt) ? at : -1;
     };
     for (int k = tid; k < 4 * a.nr; k += nt) {
         const int o = entry_cell(k);
@@ -792,6 +824,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
     using Mail = ResMail<S, (CAP > 1)>;
     const Mail mb(c);
     unsigned long long *const box = a.mail + ((long long)T.s * c.tx * c.tz + T.t) * mb.all;
+    const MailSpan shot(box - (long long)T.t * mb.all, (long long)c.tx * c.tz * mb.all, stt), mine(box, mb.all, stt);
     const ResSend<S, Mail> send(box, T, c, mb, g, e0);
     const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const qrow = q00 + e0 * PP + 4 * g;
@@ -799,6 +832,19 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
     float *const zrow = &sh.bz[e0 + 2 * M][4 * lane];
     const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
     const float2 *const cf = a.st.nc;
+#ifdef FWI_CHECKED
+    bool sound = FWI_SPAN(sh.q, qrow - (M - 1) * PP - 4, qrow + (R - 1 + M) * PP + 8, stt) &&
+                 FWI_SPAN(sh.pn[0], prow - (M - 1) * PP - 4, prow + (R - 1 + M) * PP + 8, stt) &&
+                 FWI_SPAN(sh.bz, zrow - M * PZ, zrow + (R + M - 2) * PZ + 4, stt) && in_field(e0 + M, R, S::E, stt) &&
+                 in_field(T.h + M - 1 + HR, 1, S::E + HR, stt);   // the last row of pressure fetched
+    for (int k = tid; k < recv.n; k += nt) {
+        int w, o;
+        recv.item(T, mb, k, w, o);
+        sound = FWI_SPAN(sh.q, q00 + o, q00 + o + 4, stt) && sound;
+    }
+    cp_wait<0>();
+    if (__syncthreads_or(!sound)) return;   // (the neighbours' waits for this tile expire)
+#endif
     const bool inner = e0 >= 0 && e0 + R <= T.h;
     const float *const rs = a.res + (long long)T.s * a.nr * a.nt;
     const int n4 = 4 * a.nr, nent = sh.nent;
@@ -912,13 +958,13 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
             float4 q[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) q[r] = pmul(rscale(azr[r], axv), pmul(Kv[r], pb[r]));
-            send.put(T, mb, slot, e0, q, tag);
+            send.put(T, mb, slot, e0, q, tag, shot);
             if (own)
 #pragma unroll
                 for (int r = 0; r < R; ++r)
                     if (inner || (e0 + r >= 0 && e0 + r < T.h)) st4(qrow + r * PP, q[r]);
         }
-        if (!recv.get(box + slot, T, mb, q00, tag, tid, nt, a.wait.polls)) res_expired(a.wait, stt, &sh.abort);
+        if (!recv.get(box + slot, T, mb, q00, tag, tid, nt, a.wait.polls, mine)) res_expired(a.wait, stt, &sh.abort);
         cp_wait<0>();
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
@@ -1008,7 +1054,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
         sh.si[tid] = (int)(o % d.Px) - 4 * T.g0;
         sh.sw[tid] = a.src.w[4 * T.s + tid];
     }
-    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid);
+    if (a.traces) res_receivers(sh.rec, T, d, a.ridx, a.rw, a.nr, PP, tid, S::E * PP - 8, stt);
     float *const p00 = &sh.p[HR][8], *const q00 = &sh.q[HR][8];
     if (a.p0)   // initial fields of the tile and its halo
         for (int k = tid; k < (T.h + 2 * HR) * (T.ng + 4); k += nt) {
@@ -1062,12 +1108,27 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
     const Mail mb(c);
     const long long tile = (long long)T.s * c.tx * c.tz + T.t;
     unsigned long long *const boxp = a.mail + tile * mb.all, *const boxq = a.mailq + tile * mb.all;
+    const long long words = (long long)c.tx * c.tz * mb.all;
+    const MailSpan shotp(boxp - (long long)T.t * mb.all, words, stt), shotq(boxq - (long long)T.t * mb.all, words, stt),
+        minep(boxp, mb.all, stt), mineq(boxq, mb.all, stt);
     const ResSend<S, Mail> sendp(boxp, T, c, mb, g, e0), sendq(boxq, T, c, mb, g, e0);
     const ResRecv<S, Mail> recv(T, mb, tid, nt);
     float *const prow = p00 + e0 * PP + 4 * g, *const qrow = q00 + e0 * PP + 4 * g;
     float *const vrow = &sh.vz[e0 + 2 * M][4 * lane], *const urow = &sh.uz[e0 + 2 * M][4 * lane];
     const float2 *const azr = sh.az + e0 + M, *const azhr = sh.azh + e0 + M;
     const float2 *const nc = a.st.nc;
+#ifdef FWI_CHECKED
+    bool sound = FWI_SPAN(sh.p, prow - (M - 1) * PP - 4, prow + (R - 1 + M) * PP + 8, stt) &&
+                 FWI_SPAN(sh.q, qrow - (M - 1) * PP - 4, qrow + (R - 1 + M) * PP + 8, stt) &&
+                 FWI_SPAN(sh.vz, vrow - M * PZ, vrow + (R + M - 2) * PZ + 4, stt) &&
+                 FWI_SPAN(sh.uz, urow - M * PZ, urow + (R + M - 2) * PZ + 4, stt) && in_field(e0 + M, R, S::E, stt);
+    for (int k = tid; k < recv.n; k += nt) {
+        int w, o;
+        recv.item(T, mb, k, w, o);
+        sound = FWI_SPAN(sh.p, p00 + o, p00 + o + 4, stt) && FWI_SPAN(sh.q, q00 + o, q00 + o + 4, stt) && sound;
+    }
+    if (__syncthreads_or(!sound)) return;   // (the neighbours' waits for this tile expire)
+#endif
     const bool inner = e0 >= 0 && e0 + R <= T.h;
 
     float wn = hsrc ? __ldg(a.src.wav + a.n0) : 0.f;
@@ -1172,8 +1233,8 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
                 }
             if (n + 1 < a.n1) wn = __ldg(a.src.wav + n + 1);
         }
-        sendp.put(T, mb, slot, e0, p, tag);
-        sendq.put(T, mb, slot, e0, q, tag);
+        sendp.put(T, mb, slot, e0, p, tag, shotp);
+        sendq.put(T, mb, slot, e0, q, tag, shotq);
         if (own)
 #pragma unroll
             for (int r = 0; r < R; ++r)
@@ -1187,13 +1248,14 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
 #pragma unroll
             for (int r = 0; r < R; ++r)
                 if (e0 + r == 0) v = q[r].x;
-            asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(boxq - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3)),
-                         "l"((unsigned long long)tag << 32 | __float_as_uint(v))
-                         : "memory");
+            unsigned long long *const dg = boxq - (long long)(c.tx + 1) * mb.all + 2 * mb.slot + (n & 3);
+            if (shotq.has(dg, 1))
+                asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(dg), "l"((unsigned long long)tag << 32 | __float_as_uint(v))
+                             : "memory");
         }
-        bool ok = recv.get(boxp + slot, T, mb, p00, tag, tid, nt, a.wait.polls);
-        ok = recv.get(boxq + slot, T, mb, q00, tag, tid, nt, a.wait.polls) && ok;
-        if (tid == 0 && sh.rec.diag && T.R && T.D) {
+        bool ok = recv.get(boxp + slot, T, mb, p00, tag, tid, nt, a.wait.polls, minep);
+        ok = recv.get(boxq + slot, T, mb, q00, tag, tid, nt, a.wait.polls, mineq) && ok;
+        if (tid == 0 && sh.rec.diag && T.R && T.D && mineq.has(boxq + 2 * mb.slot + (n & 3), 1)) {
             unsigned long long v = 0;
             int spin = 0;
             do {
@@ -1205,7 +1267,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_born(const __grid_constan
         if (!ok) res_expired(a.wait, stt, &sh.abort);
         __syncthreads();
         if (*reinterpret_cast<volatile int *>(&sh.abort)) break;
-        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, q00, PP, tid);
+        if (a.traces) res_sample(sh.rec, T, d, a.ridx, a.rw, a.traces, a.nr, a.nt, n, q00, PP, tid, S::E * PP - 8, stt);
         if (!own || !inner)
 #pragma unroll
             for (int r = 0; r < R; ++r)
