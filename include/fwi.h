@@ -30,8 +30,8 @@
  *  - Work on different streams must use different workspaces.
  *  - Time steps of grids that fit the GPU's registers run on chip, many steps a launch: a
  *    cooperative launch, which waits until the whole GPU can hold it, and whose blocks exchange
- *    their edges through the workspace.  The others stream through memory, a step a launch.
- *    Results are bitwise the same either way.
+ *    their edges through the workspace.  The others, and those on a stream that cannot hold such a
+ *    launch, stream through memory, a step a launch.  Results are bitwise the same either way.
  */
 #ifndef FWI_H_
 #define FWI_H_
@@ -235,6 +235,12 @@ int fwi_set_accumulation(int steps);
  * seconds).  0 expires at the first step of every launch whose shots span several blocks: the
  * way to test a caller's handling of the error. */
 int fwi_set_wait_limit(int polls);
+
+/* Most blocks of an on-chip launch that the calling thread enqueues afterwards; larger ones are
+ * refused as CUDA refuses one that its stream cannot hold (a stream of part of the GPU), and the
+ * steps stream.  Negative restores the default, no bound; 0 streams every step.  An engine tries
+ * once, with a block an SM, when its first job would step on chip. */
+int fwi_set_chip_blocks(int blocks);
 
 /* Launch-shape tuning (no counterpart in the paper: the tile-shape autotuner's hook).  By
  * default the strip height of the streaming kernels is tuned online: for each launch shape

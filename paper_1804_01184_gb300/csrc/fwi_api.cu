@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdarg>
+#include <climits>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -87,6 +88,17 @@ struct Profiler {
         kind.resize(used + 1);
         kind[used] = k;
         return &ev[2 * used++];
+    }
+    // the launch that `pair` was for did not take place
+    void drop(const cudaEvent_t *pair)
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        for (size_t k = used; k-- > 0;)
+            if (kind[k] >= 0 && &ev[2 * k] == pair) {
+                --seen[kind[k]];
+                kind[k] = -1;
+                return;
+            }
     }
 };
 Profiler g_prof;
@@ -711,14 +723,14 @@ int forward_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     ResPlan rp;
     if (res_wanted(P, RES_FWD, bg, rp)) {
         const int C = with_hist ? P.C : P.nt;
-        for (int n0 = 0; n0 < P.nt; n0 += C) {
+        int rc = FWI_OK;
+        for (int n0 = 0; n0 < P.nt && rc == FWI_OK; n0 += C) {
             const int n1 = std::min(n0 + C, P.nt);
-            const int rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, n0 / C),
-                                       n1 < P.nt ? res_checkpoint(P, work, n1 / C) : ResState{},
-                                       with_hist && n1 == P.nt ? at<float>(work, P.snap) : nullptr, traces);
-            if (rc) return rc;
+            rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, n0 / C),
+                             n1 < P.nt ? res_checkpoint(P, work, n1 / C) : ResState{},
+                             with_hist && n1 == P.nt ? at<float>(work, P.snap) : nullptr, traces);
         }
-        return FWI_OK;
+        if (rc != RES_REFUSED) return rc;   // refused: from step 0 by streaming
     }
     const int last0 = with_hist ? (P.nseg - 1) * P.C : P.nt + 1;
     float *snap = with_hist ? at<float>(work, P.snap) : nullptr;
@@ -777,7 +789,8 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const size_t bf = (size_t)bg * d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * d.Np;
     ResPlan ra;
-    const bool chip = res_wanted(P, RES_ADJ, bg, ra);
+    bool chip = res_wanted(P, RES_ADJ, bg, ra);
+    int injected = -1;            // step whose residual is in pbar although its adjoint step is not taken
     int first = P.nt & 1;         // buffers holding pbar^{nt}, vbar^{nt-1/2} = 0
     CK(cudaMemsetAsync(at<char>(work, P.ap[first]), 0, bf, st));
     CK(cudaMemsetAsync(at<char>(work, P.avx[first]), 0, bf, st));
@@ -788,15 +801,17 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
         if (k < P.nseg - 1) {   // recompute the segment from its checkpoint
             TraceRange tr(PH_RECOMPUTE);
             ResPlan rp;
-            if (res_wanted(P, RES_FWD, bg, rp)) {
-                const int rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, k), ResState{}, snap,
-                                           nullptr);
-                if (rc) return rc;
-            } else {
-                const float *ck = at<float>(work, P.ckpt) + (size_t)k * 3 * slot;
-                CK(cudaMemcpyAsync(snap, ck, bf, cudaMemcpyDeviceToDevice, st));
-                CK(cudaMemcpyAsync(at<float>(work, P.vx[n0 & 1]), ck + slot, bf, cudaMemcpyDeviceToDevice, st));
-                CK(cudaMemcpyAsync(at<float>(work, P.vz[n0 & 1]), ck + 2 * slot, bf, cudaMemcpyDeviceToDevice, st));
+            int rc = RES_REFUSED;
+            if (res_wanted(P, RES_FWD, bg, rp))
+                rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, k), ResState{}, snap, nullptr);
+            if (rc != FWI_OK && rc != RES_REFUSED) return rc;
+            if (rc == RES_REFUSED) {
+                const ResState ck = res_checkpoint(P, work, k);   // step 0: zeros, which on-chip steps do not store
+                float *const to[3] = {snap, at<float>(work, P.vx[n0 & 1]), at<float>(work, P.vz[n0 & 1])};
+                const float *const from[3] = {ck.p, ck.vx, ck.vz};
+                for (int q = 0; q < 3; ++q)
+                    CK(k == 0 ? cudaMemsetAsync(to[q], 0, bf, st)
+                              : cudaMemcpyAsync(to[q], from[q], bf, cudaMemcpyDeviceToDevice, st));
                 for (int n = n0; n < n1; ++n)
                     f.step(n, s0, bg, snap + (size_t)(n - n0) * slot, snap + (size_t)(n + 1 - n0) * slot);
             }
@@ -811,6 +826,11 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
                        at<float>(work, P.accK), snap + (size_t)(n + 1 - n0) * slot, bg, P.nr, P.nt, n, d.Np,
                        at<long long>(work, P.ridx), at<float>(work, P.rw), at<int>(work, P.rl), res);
             int rc = res_adjoint(P, work, st, ra, bg, n, lo, first, pl, res);
+            if (rc == RES_REFUSED && n == P.nt - 1) {   // the first launch: by streaming instead
+                chip = false;
+                injected = n;
+                break;
+            }
             if (rc) return rc;
             first ^= 1;
             if (lo % P.acc == 0 && (rc = flush_acc(P, work, bg, st))) return rc;
@@ -818,7 +838,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
         }
         for (int n = n1 - 1; !chip && n >= n0; --n) {
             const float *pn = snap + (size_t)(n - n0) * slot, *pn1 = snap + (size_t)(n + 1 - n0) * slot;
-            if (P.nr > 0)   // pbar^{n+1} += R^T r_n, with its K-gradient term (R^T r_n) p^{n+1}
+            if (P.nr > 0 && n != injected)   // pbar^{n+1} += R^T r_n, with its K-gradient term (R^T r_n) p^{n+1}
                 PLAUNCH(fwi::k_adj_inject_k, (bg * 4 * P.nr + 127) / 128, 128, 0, st, at<float>(work, P.ap[(n + 1) & 1]),
                        at<float>(work, P.accK), pn1, bg, P.nr, P.nt, n, d.Np, at<long long>(work, P.ridx),
                        at<float>(work, P.rw), at<int>(work, P.rl), res);
@@ -987,8 +1007,9 @@ int fwi_born(const fwi_grid *g, fwi_param pz, const float *xi_a, const float *xi
         const int s0 = gi * P.B, bg = std::min(P.B, P.ns - s0);
         ResPlan rp;
         if (res_wanted(P, RES_BORN, bg, rp)) {
-            if ((rc = res_born(P, work, st, src->wavelet, rp, s0, bg, dtraces + (size_t)s0 * P.nr * P.nt))) return rc;
-            continue;
+            rc = res_born(P, work, st, src->wavelet, rp, s0, bg, dtraces + (size_t)s0 * P.nr * P.nt);
+            if (rc == FWI_OK) continue;
+            if (rc != RES_REFUSED) return rc;
         }
         const size_t bf = (size_t)bg * d.Np * sizeof(float);
         for (size_t off : {P.p[0], P.vx[0], P.vz[0], P.dp[0], P.dvx[0], P.dvz[0]})
@@ -1182,6 +1203,13 @@ int fwi_set_wait_limit(int polls)
     return FWI_OK;
 }
 
+int fwi_set_chip_blocks(int blocks)
+{
+    g_err.clear();
+    g_chip_blocks = blocks < 0 ? INT_MAX : blocks;
+    return FWI_OK;
+}
+
 int fwi_set_accumulation(int steps)
 {
     if (steps < 0) return fail(FWI_EINVAL, "accumulation chunk must be >= 0 steps");
@@ -1215,6 +1243,7 @@ int fwi_profile_report(char *buf, size_t len)
     std::vector<long long> cnt(g_prof.names.size(), 0);
     int rc = FWI_OK;
     for (size_t k = 0; k < g_prof.used; ++k) {
+        if (g_prof.kind[k] < 0) continue;
         float t = 0.f;
         cudaError_t e = cudaEventSynchronize(g_prof.ev[2 * k + 1]);
         if (e == cudaSuccess) e = cudaEventElapsedTime(&t, g_prof.ev[2 * k], g_prof.ev[2 * k + 1]);

@@ -5,7 +5,7 @@ PyTorch supplies device memory (inputs, outputs and the scratch workspace) and s
 The functions carry the C names: ``fwi_model``, ``fwi_born``, ``fwi_adjoint``,
 ``fwi_gradient`` (optionally weighted per trace), ``fwi_misfit``, ``fwi_workspace_bytes``,
 ``fwi_status``, ``fwi_model_noalloc``, ``fwi_status_noalloc``, ``fwi_set_tile``, ``fwi_set_checkpoint``,
-``fwi_set_accumulation``, ``fwi_set_wait_limit``, ``fwi_trace``.
+``fwi_set_accumulation``, ``fwi_set_wait_limit``, ``fwi_set_chip_blocks``, ``fwi_trace``.
 
 There is no fallback: if libfwi.so has not been built (``paper_1804_01184_gb300.build``)
 or no CUDA device is present, these functions raise.
@@ -81,6 +81,7 @@ def _open(path):
     L.fwi_set_checkpoint.argtypes = [C.c_int]
     L.fwi_set_accumulation.argtypes = [C.c_int]
     L.fwi_set_wait_limit.argtypes = [C.c_int]
+    L.fwi_set_chip_blocks.argtypes = [C.c_int]
     L.fwi_trace.argtypes = [C.c_int]
     L.fwi_trace_report.argtypes = [C.c_char_p, C.c_size_t]
     L.fwi_model_noalloc.argtypes = [gp, C.c_int, vp, vp, sp, rp, vp, vp]
@@ -207,6 +208,12 @@ def fwi_set_wait_limit(polls: int = -1):
     """Polls after which a block of an on-chip launch gives up on a neighbour, for the launches
     this thread enqueues afterwards (negative: the default; 0: at once, to test error handling)."""
     _raise(lib().fwi_set_wait_limit(int(polls)))
+
+
+def fwi_set_chip_blocks(blocks: int = -1):
+    """Most blocks of the on-chip launches this thread enqueues afterwards (negative: no bound);
+    larger ones are refused and their steps stream."""
+    _raise(lib().fwi_set_chip_blocks(int(blocks)))
 
 
 def fwi_trace(enable: bool = True):
