@@ -1154,7 +1154,15 @@ int fwi_misfit_weighted(const float *traces, const float *data, long long ntrace
     cfg.numAttrs = 1;
     cudaEvent_t *ev = g_prof.next("fwi::k_misfit");
     if (ev) cudaEventRecord(ev[0], st);
-    CK(cudaLaunchKernelEx(&cfg, fwi::k_misfit, traces, data, n, weights, nt, misfit));
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fwi::k_misfit, traces, data, n, weights, nt, misfit);
+    while (e == cudaErrorInvalidClusterSize && nb > 1) {   // a stream of fewer SMs than the cluster takes
+        cudaGetLastError();
+        nb /= 2;
+        cfg.gridDim = dim3(nb);
+        attr[0].val.clusterDim = {nb, 1, 1};
+        e = cudaLaunchKernelEx(&cfg, fwi::k_misfit, traces, data, n, weights, nt, misfit);
+    }
+    CK(e);
     if (ev) cudaEventRecord(ev[1], st);
     ++g_launches;
     return finish(st);
