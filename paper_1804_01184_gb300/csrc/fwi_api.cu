@@ -721,8 +721,8 @@ int forward_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const size_t bf = (size_t)bg * P.d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * P.d.Np;   // floats between snapshot slots
     ResPlan rp;
-    if (res_wanted(P, RES_FWD, bg, rp)) {
-        const int C = with_hist ? P.C : P.nt;
+    const int C = with_hist ? P.C : P.nt;
+    if (res_wanted(P, RES_FWD, bg, C, rp)) {
         int rc = FWI_OK;
         for (int n0 = 0; n0 < P.nt && rc == FWI_OK; n0 += C) {
             const int n1 = std::min(n0 + C, P.nt);
@@ -789,7 +789,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
     const size_t bf = (size_t)bg * d.Np * sizeof(float);
     const size_t slot = (size_t)P.B * d.Np;
     ResPlan ra;
-    bool chip = res_wanted(P, RES_ADJ, bg, ra);
+    bool chip = res_wanted(P, RES_ADJ, bg, std::min(P.acc, P.C), ra);
     int injected = -1;            // step whose residual is in pbar although its adjoint step is not taken
     int first = P.nt & 1;         // buffers holding pbar^{nt}, vbar^{nt-1/2} = 0
     CK(cudaMemsetAsync(at<char>(work, P.ap[first]), 0, bf, st));
@@ -802,7 +802,7 @@ int adjoint_group(const Plan &P, void *work, cudaStream_t st, const float *wav, 
             TraceRange tr(PH_RECOMPUTE);
             ResPlan rp;
             int rc = RES_REFUSED;
-            if (res_wanted(P, RES_FWD, bg, rp))
+            if (res_wanted(P, RES_FWD, bg, P.C, rp))
                 rc = res_forward(P, work, st, wav, rp, s0, bg, n0, n1, res_checkpoint(P, work, k), ResState{}, snap, nullptr);
             if (rc != FWI_OK && rc != RES_REFUSED) return rc;
             if (rc == RES_REFUSED) {
@@ -1006,7 +1006,7 @@ int fwi_born(const fwi_grid *g, fwi_param pz, const float *xi_a, const float *xi
         TraceRange tr(PH_BORN);
         const int s0 = gi * P.B, bg = std::min(P.B, P.ns - s0);
         ResPlan rp;
-        if (res_wanted(P, RES_BORN, bg, rp)) {
+        if (res_wanted(P, RES_BORN, bg, P.nt, rp)) {
             rc = res_born(P, work, st, src->wavelet, rp, s0, bg, dtraces + (size_t)s0 * P.nr * P.nt);
             if (rc == FWI_OK) continue;
             if (rc != RES_REFUSED) return rc;
