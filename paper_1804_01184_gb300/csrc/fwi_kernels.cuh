@@ -338,10 +338,11 @@ __device__ __forceinline__ double block_sum(double v)
 // J = 1/2 sum w (tr - data)^2 in FP64 (a fixed summation order, no scratch): the least-squares
 // misfit of one set of traces (Sec. "Modelling and Inversion"), each trace (nt samples) weighted
 // by w[trace] (w null: 1).  One cluster; its blocks' sums meet in block 0's shared memory in block
-// order (a barrier that every block passes by starting, and waits for after its summation, comes
-// before: another block's shared memory is there only once that block runs).  The FP64 pipe (two lanes an SM) bounds it: a subtraction and a multiply-add an element,
-// half of the total taken at the end, over the cluster's SMs.  1.4 M elements: 106 us (1974 in one
-// block with five FP64 operations an element).
+// order.  (Another block's shared memory is there only once that block runs: all arrive at a
+// cluster barrier when they start, and wait for it after their summation.)  The FP64 pipe (two lanes
+// an SM) bounds it: a subtraction and a multiply-add an element, half of the total taken at the
+// end, over the cluster's SMs.  1.4 M elements: 106 us (1974 in one block with five FP64
+// operations an element).
 constexpr int MISFIT_NT = 512;
 
 __global__ void __launch_bounds__(MISFIT_NT) k_misfit(const float *__restrict__ tr, const float *__restrict__ data,
