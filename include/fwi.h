@@ -259,7 +259,7 @@ int fwi_set_tile(int tz, int variant);
  * problems -- shots of different surveys, line searches, sweeps over models).
  *
  * An engine owns a caller-allocated device arena (256-byte aligned; the engine never
- * allocates device memory) and one stream.  fwi_engine_submit() queues a job; jobs are
+ * allocates device memory; it takes one word of pinned host memory) and one stream.  fwi_engine_submit() queues a job; jobs are
  * admitted first-in first-out whenever their workspace (the plan the job's work_budget
  * gives) fits into the free part of the arena (first-fit), and it returns to the arena
  * when they finish, so new jobs join while earlier ones still run.

@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(32 * S::NW, 1) k_res_adj(const __grid_constant
 //
 // Background and scattered wavefields (see k_born_warp) stepped together on chip: the forward
 // kernel's structure with two of everything.  Three rows a warp; the model's perturbation sits in
-// shared memory, read by its own lane alone.  10 shots of 201^2: 6.9 us a step (two rows 7.6).
+// shared memory, read by its own lane alone.  10 shots of 201^2: 6.6 us a step (two rows 7.6).
 using ResBorn2 = ResShape<2, 3, 12>;
 using ResBorn4 = ResShape<4, 3, 12>;
 
