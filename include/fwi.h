@@ -238,8 +238,8 @@ int fwi_set_wait_limit(int polls);
 
 /* Most blocks of an on-chip launch that the calling thread enqueues afterwards; larger ones are
  * refused as CUDA refuses one that its stream cannot hold (a stream of part of the GPU), and the
- * steps stream.  Negative restores the default, no bound; 0 streams every step.  An engine tries
- * once, with a block an SM, when its first job would step on chip. */
+ * steps stream.  Negative restores the default, no bound; 0 streams every step.  An engine's
+ * launches count as a block an SM; it tries its stream once, when a job would first step on chip. */
 int fwi_set_chip_blocks(int blocks);
 
 /* Launch-shape tuning (no counterpart in the paper: the tile-shape autotuner's hook).  By

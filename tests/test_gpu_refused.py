@@ -71,3 +71,24 @@ def test_engine(F, blocks):
     assert not any("k_res_" in k for k in used), used
     got = (out[t[0]].traces, out[t[1]].misfit, out[t[1]].grads)
     assert all(torch.equal(x, y) for x, y in zip(got, ref))
+
+
+def test_engine_follows_the_bound_between_calls(F):
+    """The bound holds for the calls that follow it, also in an engine that has stepped on chip before."""
+    from paper_1804_01184_gb300 import engine
+    w = I.small_case(seed=33, nx=140, nz=120, nt=70, order=8, sponge=9, ns=3, nr=9)
+    g = gpu_grid(w)
+    ar, tail = (g, w.pz, w.xi_a, w.xi_b), (w.src_xy, w.wavelet, w.rec_xy)
+    E = engine.Engine(1 << 30)
+    out = []
+    try:
+        for blocks, on in ((-1, True), (0, False), (60, False), (-1, True)):
+            F.fwi_set_chip_blocks(blocks)
+            E.submit_model(*ar, *tail, work_budget=1 << 28)
+            (res,), used = kernels(F, lambda: E.drain(256))
+            assert any("k_res_" in k for k in used) == on, used
+            out.append(res.traces)
+    finally:
+        F.fwi_set_chip_blocks(-1)
+        E.close()
+    assert all(torch.equal(x, out[0]) for x in out[1:])
