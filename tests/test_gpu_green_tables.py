@@ -49,12 +49,15 @@ CASES = {
     "paper": dict(nx=121, nz=121, dx=5.0, src=ring(10, 490.0), rec=ring(100, 490.0, 0.5), f=0.25 * np.arange(1, 61), radial=1, near=0),
     "near and far nodes": dict(nx=60, nz=41, dx=5.0, src=ring(4, 195.0), rec=ring(20, 195.0, 0.5), f=0.4 * np.arange(1, 34), radial=1, near=1),
     "few frequencies": dict(nx=61, nz=33, dx=5.0, src=ring(3, 190.0), rec=ring(9, 190.0, 0.5), f=3.0 * np.arange(1, 6), radial=1, near=1),
+    "few frequencies, more points": dict(nx=61, nz=33, dx=5.0, src=ring(6, 190.0), rec=ring(19, 200.0, 0.5), f=3.0 * np.arange(1, 6), radial=1, near=1),
+    "the highest wavenumber of an interval": dict(nx=80, nz=60, dx=0.8, src=ring(5, 54.0), rec=ring(14, 55.0, 0.5), f=np.linspace(0.7, 19.89, 40), radial=1, near=1),
     "four decades of frequency": dict(nx=90, nz=64, dx=4.0, src=ring(5, 235.0), rec=ring(30, 240.0, 0.5), f=np.geomspace(0.002, 14.0, 37), radial=1, near=1),
     # the table of all frequencies does not fit the scratch: two frequency blocks
     "frequency blocks": dict(nx=9, nz=121, dx=5.0, src=ring(3, 360.0), rec=ring(7, 370.0, 0.5), f=0.25 * np.arange(1, 61), radial=2, near=0),
     # distances that are whole intervals (h = 1): both sides of an interval's edge and of the first one
     "interval edges": dict(nx=200, nz=40, dx=1.0, x0=0.0, z0=0.0, src=np.array([[-3.0, 0.0], [-40.0, 5.0]], np.float32),
-                           rec=np.array([[203.0, 0.0], [-64.0, 3.0], [-63.0, 7.0], [230.0, 39.0]], np.float32), f=0.5 * np.arange(1, 31), radial=1, near=1),
+                           rec=np.array([[203.0, 0.0], [-64.0, 3.0], [-63.0, 7.0], [230.0, 39.0], [-32.0, 1.0], [-31.0, 9.0]], np.float32),
+                           f=0.5 * np.arange(1, 31), radial=1, near=1),
     # wavenumbers whose pairs FP32 does not hold
     "seven decades of frequency": dict(nx=60, nz=41, dx=5.0, src=ring(2, 195.0), rec=ring(8, 195.0, 0.5), f=np.geomspace(1e-6, 13.0, 33), radial=0, near=1),
     "every node near": dict(nx=40, nz=40, dx=5.0, src=ring(2, 160.0), rec=ring(6, 160.0, 0.5), f=0.01 * np.arange(1, 3), radial=0, near=1),
